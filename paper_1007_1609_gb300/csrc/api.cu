@@ -125,6 +125,8 @@ struct cbdg_lattice {
   DBuf sym_rep, sym_list;  // cbdg_set_symmetry: representative of every site, distinct representatives
   int sym_n = 0;           // number of representatives (0: no symmetry reduction)
   int site_cpl = 0;      // 1 while cpl replaces the scalar coupling
+  bool uniform = false;  // every bond of the lattice has the same real hopping, hop_all
+  double hop_all = 0.0;
   const double *coupling_site() const { return site_cpl ? static_cast<const double *>(cpl.p) : nullptr; }
   // options
   int K = 65536;
@@ -447,6 +449,48 @@ cbdg_status run_columns(cbdg_lattice *L, const int32_t *sites, int n_sites, int 
   int want_split = static_cast<int>(L->row_split), want_depth = static_cast<int>(L->depth);
   const bool cplx_multi = mode != kReal && use_cplx_multi(L);
   if (cplx_multi) W = 2;
+  // real FP32 lattices with one hopping: the whole recursion in the registers
+  // of thread-block clusters, one launch
+  ClusterPlan plan;
+  if (mode == kReal && L->precision == CBDG_FP32_MIXED && L->uniform && L->resident && L->slab_w == 0 &&
+      L->row_split == 0 && L->depth == 0 && L->temporal == 0 && !L->autotune && !L->stall && n_sites > 0 &&
+      plan_cluster(L->Lx, L->Ly, n_sites, &plan)) {
+    CK(L->acc_n.ensure(static_cast<size_t>(n_sites) * sizeof(double)));
+    CK(L->acc_d.ensure(static_cast<size_t>(n_sites) * 4 * sizeof(double2)));
+    ClusterArgs c{};
+    c.params = L->params.as<float>();
+    c.scal = L->scal.as<double>();
+    c.C = L->C.as<double>();
+    c.eps = L->eps.as<double>();
+    c.delta = L->delta.as<double2>();
+    c.sites = sites;
+    c.acc_n = L->acc_n.as<double>();
+    c.acc_d = L->acc_d.as<double2>();
+    c.mu_ee = mom_ee;
+    c.mu_eh = mom_eh;
+    c.flags = L->flags.as<unsigned int>();
+    c.mu = L->mu;
+    c.hop = L->hop_all;
+    c.tol = 1e-4;
+    c.Lx = L->Lx;
+    c.Ly = L->Ly;
+    c.px = L->px;
+    c.py = L->py;
+    c.ncols = n_sites;
+    c.M = M;
+    c.steps = (M + 1) / 2 - 1;
+    c.mom_stride = mom_stride;
+    CK(launch_cluster(c, plan, L->stream));
+    L->launches += 1;
+    if (finalize) {
+      CK(launch_finalize_onsite(n_sites, sites, L->coupling, L->coupling_site(), L->acc_n.as<double>(),
+                                L->acc_d.as<double2>(), L->dout.as<double2>(), L->nout.as<double>(), L->stream));
+      L->launches += 1;
+    }
+    L->last_cfg = StepConfig{1, 0, 1, plan.threads, 0};  // depth 0: on chip
+    L->last_temporal = 1;
+    return CBDG_OK;
+  }
   // small real lattices: the whole recursion in shared memory, one launch
   const int Wres = (mode == kReal && L->resident && L->slab_w == 0 && L->row_split == 0 && L->depth == 0 &&
                     !L->autotune && !L->stall)
@@ -1247,6 +1291,21 @@ cbdg_status check_hop(const cbdg_lattice_desc *d, const std::vector<cbdg_complex
       if (z.im != 0.0) return fail(CBDG_ERR_INVALID_ARG, "complex hop with complex_field = 0");
   return CBDG_OK;
 }
+// Whether every bond inside the lattice has the same real hopping *t (0 where
+// the lattice has no bond).
+bool uniform_hop(const cbdg_lattice_desc *d, const std::vector<cbdg_complex> &hop, double *t) {
+  bool any = false;
+  *t = 0.0;
+  for (int i = 0; i < d->Lx * d->Ly; ++i)
+    for (int dir = 0; dir < d->n_dirs; ++dir) {
+      if (host_neighbour(d, i, dir) < 0) continue;
+      const cbdg_complex z = hop[static_cast<size_t>(i) * d->n_dirs + dir];
+      if (!any) *t = z.re;
+      any = true;
+      if (z.im != 0.0 || z.re != *t) return false;
+    }
+  return true;
+}
 // Adjoint of one self-consistency map for general lattices (complex vectors:
 // Peierls hoppings, next-nearest neighbours, on-site or bond pairing), with
 // g = dL/dRe Delta_out + i dL/dIm Delta_out [nd] already in L->adj_wc
@@ -1482,6 +1541,7 @@ cbdg_status cbdg_build_lattice(const cbdg_lattice_desc *d, cbdg_stream stream,
   L->mu = d->mu;
   L->coupling = d->coupling;
   L->nd = nd;
+  L->uniform = uniform_hop(d, hop, &L->hop_all);
   auto bail = [&](cudaError_t err, const char *what) {
     cbdg_status st = cuda_fail(err, what);
     cbdg_destroy(L);
@@ -2144,10 +2204,10 @@ cbdg_status cbdg_set_hamiltonian(cbdg_lattice *L, const double *eps, const cbdg_
     for (int i = 0; i < L->N; ++i)
       if (!isfinite(he[i])) return fail(CBDG_ERR_INVALID_ARG, "eps[%d] is not finite", i);
   }
+  cbdg_lattice_desc d{};
   if (hop) {
     cudaError_t e = host_copy(hop, static_cast<size_t>(L->N) * L->n_dirs, hh);
     if (e != cudaSuccess) return cuda_fail(e, "reading hop");
-    cbdg_lattice_desc d{};
     d.Lx = L->Lx;
     d.Ly = L->Ly;
     d.periodic_x = L->px;
@@ -2159,8 +2219,14 @@ cbdg_status cbdg_set_hamiltonian(cbdg_lattice *L, const double *eps, const cbdg_
   }
   // validated host copies: upload (nothing changes on an invalid call)
   if (eps) CK(cudaMemcpyAsync(L->eps.p, he.data(), L->N * sizeof(double), cudaMemcpyHostToDevice, L->stream));
-  if (hop)
+  if (hop) {
     CK(cudaMemcpyAsync(L->hop.p, hh.data(), hh.size() * sizeof(double2), cudaMemcpyHostToDevice, L->stream));
+    double t = 0.0;
+    const bool u = uniform_hop(&d, hh, &t);
+    if (u != L->uniform || t != L->hop_all) L->drop_graph();  // the captured launch carries the hopping
+    L->uniform = u;
+    L->hop_all = t;
+  }
   CK(cudaStreamSynchronize(L->stream));
   return CBDG_OK;
 }

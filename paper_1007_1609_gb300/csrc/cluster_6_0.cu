@@ -1,0 +1,10 @@
+// The register-resident recursion (cluster.cuh): tiles 4 x 6, covering the lattice exactly.
+#include "cluster.cuh"
+
+namespace cbdg {
+
+cudaError_t launch_cluster_6_0(const ClusterArgs &a, const ClusterPlan &p, cudaStream_t s) {
+  return launch_one<6, 0>(a, p, s);
+}
+
+}  // namespace cbdg

@@ -1,0 +1,10 @@
+// The register-resident recursion (cluster.cuh): tiles 4 x 8, sticking out over open edges.
+#include "cluster.cuh"
+
+namespace cbdg {
+
+cudaError_t launch_cluster_8_1(const ClusterArgs &a, const ClusterPlan &p, cudaStream_t s) {
+  return launch_one<8, 1>(a, p, s);
+}
+
+}  // namespace cbdg

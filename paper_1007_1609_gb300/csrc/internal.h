@@ -142,6 +142,32 @@ cudaError_t launch_resident(int precision, int W, int Lx, int Ly, int ld, int nc
                             double *mu_ee, double2 *mu_eh, int mom_stride, unsigned int *flags, double tol,
                             cudaStream_t s);
 
+// The whole recursion in the registers of thread-block clusters (cluster.cu).
+constexpr int kMaxCluster = 8;
+constexpr int kClusterSmem = 226 * 1024;  // dynamic shared memory a CTA may ask for
+constexpr int kClusterBatch = 16;         // steps between two folds of the column sums
+struct ClusterArgs {
+  const float *params;     // [N][kParamStride]
+  const double *scal, *C;  // rescale, coefficient table [M]
+  const double *eps;
+  const double2 *delta;
+  const int32_t *sites;    // [ncols] start sites
+  double *acc_n;           // [ncols]
+  double2 *acc_d;          // [ncols]
+  double *mu_ee;           // [ncols][M] or null
+  double2 *mu_eh;          // [ncols][M][mom_stride] or null
+  unsigned int *flags;
+  double mu, hop, tol;     // hop: t of every bond
+  int Lx, Ly, px, py, ncols, M, steps, mom_stride;
+  int cluster, rows;       // CTAs per cluster, tile rows per CTA
+};
+struct ClusterPlan {
+  int by, cluster, rows, threads;
+  size_t smem;
+};
+bool plan_cluster(int Lx, int Ly, int ncols, ClusterPlan *p);
+cudaError_t launch_cluster(ClusterArgs a, const ClusterPlan &p, cudaStream_t s);
+
 // Recursion step for the general lattice (complex vectors; nnn: 8 hopping
 // directions; bond: nearest-neighbour pairing, which skips the column sums).
 // The partial sums, when formed, are [row_split][4][ld].

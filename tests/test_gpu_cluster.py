@@ -1,0 +1,85 @@
+"""The register-resident recursion of thread-block clusters (FP32 real on-site
+lattices with one hopping): moments and order parameter against the FP64
+oracle at the edges of its tiles (4 sites wide, 4, 6 or 8 high), of its CTAs
+and of its clusters, for every kind of edge, few and many start sites; the
+lattices it does not take (hoppings that differ) against the streamed kernels.
+Tolerances are those of the FP32 recursion: its column sums carry at most
+38 * 2^-24 of the sum of magnitudes (<= 1), doubled in a moment: 4.5e-6."""
+import numpy as np
+import pytest
+
+from oracle import oracle as orc
+from paper_1007_1609_gb300 import cbdg
+from paper_1007_1609_gb300 import workloads as wl
+from tests._common import as_oracle, gpu_available, max_abs
+from tests.test_gpu_parity import K, TOL, gpu_lattice
+
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not gpu_available(), reason="needs a CUDA GPU")]
+
+
+def lattice(Lx, Ly, px, py, M, seed):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    N = Lx * Ly
+    return wl.Problem(name=f"c{Lx}x{Ly}", Lx=Lx, Ly=Ly, periodic_x=px, periodic_y=py,
+                      eps=rng.uniform(-0.5, 0.5, size=N), mu=-0.5, hop=wl.square_hops(Lx, Ly, px, py),
+                      pairing=wl.ONSITE, coupling=2.0, delta0=rng.uniform(0.2, 0.8, size=N).astype(np.complex128),
+                      T=0.02, M=M)
+
+
+@pytest.mark.parametrize("px,py", [(0, 0), (1, 0), (0, 1), (1, 1)])
+@pytest.mark.parametrize("shape", [(3, 3, 2), (4, 8, 3), (5, 9, 37), (33, 49, 68), (65, 66, 35), (97, 95, 34),
+                                   (130, 127, 36), (256, 250, 20)])
+def test_moments_match_oracle(shape, px, py):
+    Lx, Ly, M = shape
+    p = lattice(Lx, Ly, px, py, M, seed=Lx * 13 + Ly)
+    sites = np.arange(p.N, dtype=np.int32)
+    if p.N > 64:
+        rng = np.random.default_rng(Ly)
+        sites = np.concatenate([[0, Lx - 1, p.N - Lx, p.N - 1], rng.choice(p.N, 20)]).astype(np.int32)
+    lat = gpu_lattice(p, "fp32")
+    ee, eh = lat.moments(sites, M)
+    assert lat.last_tile()[:2] == (1, 0)  # on chip, one column at a time
+    oee, oeh = orc.moments(as_oracle(p), lat.rescale, sites, M)
+    assert max_abs(ee, oee) < TOL["fp32"][0] and max_abs(eh, oeh) < TOL["fp32"][0]
+    one = lat.moments(sites[-1:], M)  # a single start site, another plan
+    assert max_abs(one[0], oee[-1:]) < TOL["fp32"][0] and max_abs(one[1], oeh[-1:]) < TOL["fp32"][0]
+
+
+@pytest.mark.parametrize("shape", [(31, 30, 0, 0, 34), (22, 37, 1, 1, 67)])
+def test_order_parameter_matches_oracle(shape):
+    Lx, Ly, px, py, M = shape
+    p = lattice(Lx, Ly, px, py, M, seed=5)
+    lat = gpu_lattice(p, "fp32")
+    d, n = lat.order_parameter(p.T, M)
+    od, on = orc.order_parameter(as_oracle(p), lat.rescale, p.T, M, K)
+    assert max_abs(d, od) < TOL["fp32"][1] and max_abs(n, on) < TOL["fp32"][1]
+
+
+def test_hoppings_that_differ_take_the_general_path():
+    """A lattice whose hoppings differ keeps the kernels that read each one;
+    replacing the hoppings moves the lattice from one path to the other, also
+    between replays of a captured iteration."""
+    p = lattice(30, 70, 0, 0, 40, seed=6)
+    q = lattice(30, 70, 0, 0, 40, seed=6)
+    q.hop = p.hop.copy()
+    q.hop[31, 0] = q.hop[32, 1] = 0.7  # the bond between sites 31 and 32
+    lat = gpu_lattice(p, "fp32")
+    for hop, prob in ((p.hop, p), (q.hop, q), (p.hop, p), (0.5 * p.hop, None)):
+        cbdg.cbdg_set_hamiltonian(lat.handle, None, np.ascontiguousarray(hop))
+        if prob is None:
+            prob = lattice(30, 70, 0, 0, 40, seed=6)
+            prob.hop = 0.5 * p.hop
+        lat.delta = prob.delta0
+        for _ in range(3):
+            lat.scf_step(prob.T, prob.M, 0.5)
+        ref, _, _, _ = orc.scf(as_oracle(prob), prob.T, prob.M, K, 0.5, 0.0, 3)
+        assert max_abs(lat.delta, ref) < TOL["fp32"][1]
+
+
+def test_spectrum_violation_is_reported():
+    p = lattice(40, 40, 0, 0, 64, seed=7)
+    lat = gpu_lattice(p, "fp32", fixed_rescale_pico=int(0.5e12))  # a far inside the band
+    with pytest.raises(cbdg.CbdgError) as ei:
+        lat.moments(np.arange(p.N, dtype=np.int32), p.M)
+    assert ei.value.status == cbdg.CBDG_ERR_SPECTRUM
