@@ -162,6 +162,11 @@ struct cbdg_lattice {
   }
 };
 
+bool cbdg_internal_uniform_hop(const cbdg_lattice *lat, double *t) {
+  *t = lat->hop_all;
+  return lat->uniform;
+}
+
 namespace {
 
 // Copies device src into a caller array (host or device).

@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
   using Rec = Record<BY>;
   using Tile = F2[BY][2];
   constexpr bool EREG = BY == 8;  // 2 (eps - mu) / a in registers, else in the thread's record
+  if (a.done && *a.done) return;  // a converged member of an ensemble: nothing to do, for every thread
   extern __shared__ __align__(16) unsigned char raw[];
   __shared__ __align__(8) unsigned long long bars[2];
   __shared__ double share[kBatch][2], col_m1, col_dl;  // the column's fold, by step modulo kBatch
@@ -458,7 +459,7 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
   for (int col = cid; col < a.ncols; col += ncl) {
     Tile pu, pv, qu, qv;  // j_{n-1}, j_n
     {
-      const int site = a.sites[col];
+      const int site = a.sites ? a.sites[col] : col;
       const double am = a.scal[kScalA];
       const double m1 = (a.eps[site] - a.mu) / am, dl = a.delta[site].x / am;
       if (t == 0) {
@@ -514,8 +515,15 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
         an += share[i][0];
         ad += share[i][1];
       }
-      a.acc_n[col] = an - (c0 + c1 * col_m1);
-      a.acc_d[col] = make_double2(ad + c1 * col_dl, 0.0);
+      an -= c0 + c1 * col_m1;
+      ad += c1 * col_dl;
+      if (a.dout) {
+        a.dout[col] = make_double2(0.5 * a.coupling * ad, 0.0);
+        a.nout[col] = 1.0 + an;
+      } else {
+        a.acc_n[col] = an;
+        a.acc_d[col] = make_double2(ad, 0.0);
+      }
       if (a.mu_ee) {
         a.mu_ee[static_cast<size_t>(col) * a.M] = 1.0;
         a.mu_ee[static_cast<size_t>(col) * a.M + 1] = col_m1;

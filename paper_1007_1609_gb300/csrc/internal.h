@@ -151,13 +151,16 @@ struct ClusterArgs {
   const double *scal, *C;  // rescale, coefficient table [M]
   const double *eps;
   const double2 *delta;
-  const int32_t *sites;    // [ncols] start sites
+  const int32_t *sites;    // [ncols] start sites, or null: 0 .. ncols - 1
   double *acc_n;           // [ncols]
   double2 *acc_d;          // [ncols]
+  const int *done;         // a member of an ensemble: its converged flag,
+  double2 *dout;           // Delta_out and n [ncols] in place of acc_n and acc_d
+  double *nout;
   double *mu_ee;           // [ncols][M] or null
   double2 *mu_eh;          // [ncols][M][mom_stride] or null
   unsigned int *flags;
-  double mu, hop, tol;     // hop: t of every bond
+  double mu, coupling, hop, tol;  // hop: t of every bond; coupling: for dout
   int Lx, Ly, px, py, ncols, M, steps, mom_stride;
   int cluster, rows;       // CTAs per cluster, tile rows per CTA
 };
@@ -342,3 +345,6 @@ cudaError_t launch_ldos_weights(int n_E, int M, int ld, int kernel, double lambd
 
 // Records msg as the calling thread's cbdg_last_error() text.
 void cbdg_internal_set_error(const char *msg);
+// Whether every bond of the lattice has the same real hopping *t.
+struct cbdg_lattice;
+bool cbdg_internal_uniform_hop(const cbdg_lattice *lat, double *t);

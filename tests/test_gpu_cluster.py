@@ -83,3 +83,19 @@ def test_spectrum_violation_is_reported():
     with pytest.raises(cbdg.CbdgError) as ei:
         lat.moments(np.arange(p.N, dtype=np.int32), p.M)
     assert ei.value.status == cbdg.CBDG_ERR_SPECTRUM
+
+
+def test_ensemble_mixes_both_kernels():
+    """Members with one hopping run in cluster registers, a member whose
+    hoppings differ in the streaming kernel; all follow the oracle's loop."""
+    ps = [lattice(24, 40, 0, 0, 48, seed=8), lattice(33, 21, 0, 0, 48, seed=9), lattice(40, 26, 0, 0, 48, seed=10)]
+    ps[1].hop = ps[1].hop.copy()
+    ps[1].hop[5, 0] = ps[1].hop[6, 1] = 1.3
+    ens = cbdg.Ensemble(ps)
+    ens.set_option(cbdg.CBDG_OPT_QUADRATURE_NODES, K)
+    _, it, _ = ens.scf(0.02, 48, 0.5, 0.0, 2)
+    assert it == 2
+    for k, p in enumerate(ps):
+        ref, _, _, _ = orc.scf(as_oracle(p), 0.02, 48, K, 0.5, 0.0, 2)
+        assert max_abs(ens.delta(k), ref) < TOL["fp32"][1]
+    ens.close()
