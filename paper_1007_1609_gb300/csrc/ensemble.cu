@@ -1,7 +1,6 @@
 // ensemble.cu -- many independent disorder realisations of uneven lattice
-// size, each iterated to self-consistency (paragraph after Eq. 20), with one
-// persistent recursion launch per iteration and the iteration captured once
-// as a CUDA graph and replayed.
+// size, each iterated to self-consistency (paragraph after Eq. 20), the iteration
+// captured once as a CUDA graph and replayed.
 //
 // Members with one hopping amplitude on every bond run in the registers of
 // thread-block clusters (cluster.cuh): one launch per member, spread over eight
@@ -12,8 +11,8 @@
 // launch over all members, the lattice changing inside the column loop, took
 // 2.10 s: the compiler then spends a quarter more instructions on a step.)
 //
-// The remaining members go to the streaming kernel.  Its
-work items are (sample, column slab of W start vectors), ordered largest
+// The remaining members go to the streaming kernel, one persistent launch per
+// iteration.  Its work items are (sample, column slab of W start vectors), ordered largest
 // sample first and handed out through an atomic counter.  A CTA owns an item
 // from j_0 to the last moment: its two vectors live in a per-CTA scratch
 // block (slab-blocked [2N][W], electron rows then hole rows per lattice row),
