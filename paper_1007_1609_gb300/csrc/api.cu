@@ -459,7 +459,7 @@ cbdg_status run_columns(cbdg_lattice *L, const int32_t *sites, int n_sites, int 
   ClusterPlan plan;
   if (mode == kReal && L->precision == CBDG_FP32_MIXED && L->uniform && L->resident && L->slab_w == 0 &&
       L->row_split == 0 && L->depth == 0 && L->temporal == 0 && !L->autotune && !L->stall && n_sites > 0 &&
-      plan_cluster(L->Lx, L->Ly, n_sites, &plan)) {
+      plan_cluster(L->Lx, L->Ly, L->px, L->py, n_sites, &plan)) {
     CK(L->acc_n.ensure(static_cast<size_t>(n_sites) * sizeof(double)));
     CK(L->acc_d.ensure(static_cast<size_t>(n_sites) * 4 * sizeof(double2)));
     ClusterArgs c{};

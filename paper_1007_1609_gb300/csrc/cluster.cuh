@@ -5,8 +5,8 @@
 // A step over vectors in HBM moves 3 streams (4 per three steps in the
 // multi-step pass), 175 KB per vector-step of the 128 x 128 lattice; here
 // nothing moves: a thread keeps j_{n-1} and j_n of a tile of 4 x BY sites of one
-// start vector in registers, an SM about 8200 sites, and a cluster of up to
-// eight CTAs one start vector of up to 65536 sites.  Clusters are persistent and
+// start vector in registers, an SM 8192 to 10240 sites, and a cluster of up
+// to sixteen CTAs one start vector of up to 163840 sites.  Clusters are persistent and
 // take one start vector after the other through all its steps.  Per step a
 // thread computes its tile (packed FP32 pairs along x), publishes the tile's
 // edge rows and columns in shared memory (the rows at a CTA's ends also in the
@@ -124,20 +124,21 @@ __device__ __forceinline__ void put(F2 (&z)[BY][2], int r, int c, float x) {
 }
 
 // Shared memory of a CTA: one record of kQuads quads (16 bytes) per thread, one
-// per tile column for the rows that the CTAs below and above push, and one of
-// zeros.  A record holds, twice (the edges of j_n and of j_{n+1}), u and v of the
+// per kGhosts tile columns for the rows that the CTAs below and above push (top
+// and bottom quads of tile column x at quad 4 (x mod kGhosts)), and one of zeros.  A record holds, twice (the edges of j_n and of j_{n+1}), u and v of the
 // tile's top and bottom sites and its left and right sites as (u, u, v, v) of
 // rows 1 and 2, 3 and 4, .. and last of rows 0 and BY - 1; then, where the
-// registers have no room for them (BY < 8), the rows of 2 (eps - mu) / a.  An odd
+// registers have no room for them (BY other than 8), the rows of 2 (eps - mu) / a.  An odd
 // number of quads keeps the accesses of neighbouring threads free of conflicts.
 template <int BY>
 struct Record {
   static constexpr int kTop = 0, kBottom = 2, kLeft = 4, kRight = 4 + BY / 2, kEdges = 4 + BY;
   static constexpr int kPar = 2 * kEdges;
-  static constexpr int kQuads = (kPar + (BY < 8 ? BY : 0)) | 1;
+  static constexpr int kQuads = (kPar + (BY != 8 ? BY : 0)) | 1;
   static constexpr int kBytes = kQuads * 16;
+  static constexpr int kGhosts = kEdges / 4;
   static constexpr int kBuffer = kEdges * 16;  // from one set of edges to the other
-  // threads an SM's registers allow (BY = 4: 128 registers a thread, 6: 168, 8: 255)
+  // threads an SM's registers allow (BY = 4: 128 registers a thread, 6: 168, 8 and 10: 255)
   static constexpr int kThreads = BY == 4 ? 512 : BY == 6 ? 384 : 256;
 };
 
@@ -156,7 +157,7 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
   const int CS = a.cluster, rank = CS > 1 ? static_cast<int>(cluster_rank()) : 0;
   const int cid = blockIdx.x / CS, ncl = gridDim.x / CS;
   const int Lx = a.Lx, Ly = a.Ly, TX = (Lx + kB - 1) / kB, TY = (Ly + BY - 1) / BY, R = a.rows;
-  const int ghost = blockDim.x, nil = ghost + (CS > 1 ? TX : 0);  // records
+  const int ghost = blockDim.x, nil = ghost + (CS > 1 ? (TX + Rec::kGhosts - 1) / Rec::kGhosts : 0);  // records
   double *xsum = reinterpret_cast<double *>(raw + (nil + 1) * Rec::kBytes);  // rank 0: [CS][3 kBatch] sums of a batch
   float *ring = reinterpret_cast<float *>(xsum + CS * 3 * kBatch);           // [2 kBatch][3][nw] warp sums of the last steps
   const unsigned e0 = smem_addr(raw);
@@ -210,28 +211,24 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
 
   // where the four neighbour tiles' edges are read
   auto record = [&](int k, int quad) { return e0 + k * Rec::kBytes + quad * 16; };
+  auto pushed = [&](int x, int quad) { return record(ghost + x / Rec::kGhosts, x % Rec::kGhosts * 4 + quad); };
   unsigned up = record(nil, 0), dn = up, lf = up, rt = up, push_up = 0, push_dn = 0;
   const unsigned own = record(t, 0);
   if (act) {
     if (tyl + 1 < rows_here) up = record(t + TX, Rec::kBottom);
-    else if (CS > 1 && (ty + 1 < TY || a.py)) up = record(ghost + tx, Rec::kBottom);
+    else if (CS > 1 && (ty + 1 < TY || a.py)) up = pushed(tx, Rec::kBottom);
     else if (a.py) up = record(tx, Rec::kBottom);
     if (tyl > 0) dn = record(t - TX, Rec::kTop);
-    else if (CS > 1 && (ty > 0 || a.py)) dn = record(ghost + tx, Rec::kTop);
+    else if (CS > 1 && (ty > 0 || a.py)) dn = pushed(tx, Rec::kTop);
     else if (a.py) dn = record((TY - 1) * TX + tx, Rec::kTop);
     if (tx > 0) lf = record(t - 1, Rec::kRight);
     else if (a.px) lf = record(t + TX - 1, Rec::kRight);
     if (tx + 1 < TX) rt = record(t + 1, Rec::kLeft);
     else if (a.px) rt = record(t - TX + 1, Rec::kLeft);
     if (CS > 1) {
-      if (tyl + 1 == rows_here && (ty + 1 < TY || a.py)) {
-        const int to = rank + 1 < CS ? rank + 1 : 0;
-        push_up = remote(e0 + (ghost + tx) * Rec::kBytes + Rec::kTop * 16, to);
-      }
-      if (tyl == 0 && (ty > 0 || a.py)) {
-        const int to = rank > 0 ? rank - 1 : CS - 1;
-        push_dn = remote(e0 + (ghost + tx) * Rec::kBytes + Rec::kBottom * 16, to);
-      }
+      if (tyl + 1 == rows_here && (ty + 1 < TY || a.py))
+        push_up = remote(pushed(tx, Rec::kTop), rank + 1 < CS ? rank + 1 : 0);
+      if (tyl == 0 && (ty > 0 || a.py)) push_dn = remote(pushed(tx, Rec::kBottom), rank > 0 ? rank - 1 : CS - 1);
     }
   }
 
@@ -539,38 +536,54 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
 }
 
 template <int BY, int RAG>
-cudaError_t launch_one(const ClusterArgs &a, const ClusterPlan &p, cudaStream_t s) {
-  auto k = cluster_kernel<BY, RAG>;
+struct Launch {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = p.cluster;
-  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cfg.blockDim = dim3(p.threads);
-  cfg.dynamicSmemBytes = p.smem;
-  cfg.stream = s;
-  // clusters that fit on the device at once, by device, cluster, CTA size and shared memory
-  static std::mutex mutex;
-  static std::map<std::tuple<int, int, int, size_t>, int> fit;
-  int dev = 0, resident = 0;
-  cudaGetDevice(&dev);
-  {
-    std::lock_guard<std::mutex> lock(mutex);
-    int &f = fit[{dev, p.cluster, p.threads, p.smem}];
-    if (f == 0) {
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kClusterSmem);
-      if (e != cudaSuccess) return e;
-      cfg.gridDim = dim3(p.cluster);
-      e = cudaOccupancyMaxActiveClusters(&f, k, &cfg);
-      if (e != cudaSuccess) return e;
-      if (f < 1) return cudaErrorInvalidConfiguration;
-    }
-    resident = f;
+  explicit Launch(const ClusterPlan &p) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = p.cluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3(p.cluster);
+    cfg.blockDim = dim3(p.threads);
+    cfg.dynamicSmemBytes = p.smem;
   }
-  cfg.gridDim = dim3(std::min(resident, a.ncols) * p.cluster);
-  return cudaLaunchKernelEx(&cfg, k, a);
+};
+
+// Clusters of the plan's shape that the current device holds at once (0: none).
+template <int BY, int RAG>
+int slots_one(const ClusterPlan &p) {
+  static std::mutex mutex;
+  static std::map<std::tuple<int, int, int, size_t>, int> known;  // by device, cluster, CTA size and shared memory
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lock(mutex);
+  const auto key = std::make_tuple(dev, p.cluster, p.threads, p.smem);
+  const auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  auto k = cluster_kernel<BY, RAG>;
+  Launch<BY, RAG> l(p);
+  int n = 0;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kClusterSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k, &l.cfg);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  known[key] = n;
+  return n;
+}
+
+template <int BY, int RAG>
+cudaError_t launch_one(const ClusterArgs &a, const ClusterPlan &p, cudaStream_t s) {
+  const int slots = slots_one<BY, RAG>(p);  // sets the kernel's attributes on the first call
+  if (slots < 1) return cudaErrorInvalidConfiguration;
+  Launch<BY, RAG> l(p);
+  l.cfg.gridDim = dim3(std::min(slots, a.ncols) * p.cluster);
+  l.cfg.stream = s;
+  return cudaLaunchKernelEx(&l.cfg, cluster_kernel<BY, RAG>, a);
 }
 
 }  // namespace

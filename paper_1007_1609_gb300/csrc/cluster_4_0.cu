@@ -7,4 +7,6 @@ cudaError_t launch_cluster_4_0(const ClusterArgs &a, const ClusterPlan &p, cudaS
   return launch_one<4, 0>(a, p, s);
 }
 
+int cluster_slots_4_0(const ClusterPlan &p) { return slots_one<4, 0>(p); }
+
 }  // namespace cbdg

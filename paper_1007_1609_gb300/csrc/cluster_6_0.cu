@@ -7,4 +7,6 @@ cudaError_t launch_cluster_6_0(const ClusterArgs &a, const ClusterPlan &p, cudaS
   return launch_one<6, 0>(a, p, s);
 }
 
+int cluster_slots_6_0(const ClusterPlan &p) { return slots_one<6, 0>(p); }
+
 }  // namespace cbdg

@@ -7,4 +7,6 @@ cudaError_t launch_cluster_8_0(const ClusterArgs &a, const ClusterPlan &p, cudaS
   return launch_one<8, 0>(a, p, s);
 }
 
+int cluster_slots_8_0(const ClusterPlan &p) { return slots_one<8, 0>(p); }
+
 }  // namespace cbdg

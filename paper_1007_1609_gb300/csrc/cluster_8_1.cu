@@ -7,4 +7,6 @@ cudaError_t launch_cluster_8_1(const ClusterArgs &a, const ClusterPlan &p, cudaS
   return launch_one<8, 1>(a, p, s);
 }
 
+int cluster_slots_8_1(const ClusterPlan &p) { return slots_one<8, 1>(p); }
+
 }  // namespace cbdg

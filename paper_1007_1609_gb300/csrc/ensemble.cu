@@ -795,7 +795,7 @@ cbdg_status cbdg_build_ensemble(const cbdg_lattice_desc *descs, int32_t n, cbdg_
   std::vector<char> resident(n, 0);
   for (int s : order) {
     ClusterPlan plan;
-    if (!uniform[s] || !plan_cluster(e->hLx[s], e->hLy[s], 1 << 20, &plan)) continue;
+    if (!uniform[s] || !plan_cluster(e->hLx[s], e->hLy[s], 0, 0, 1 << 20, &plan)) continue;
     resident[s] = 1;
     e->members.push_back({s, hop[s], plan});
   }

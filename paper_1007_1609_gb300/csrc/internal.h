@@ -143,7 +143,7 @@ cudaError_t launch_resident(int precision, int W, int Lx, int Ly, int ld, int nc
                             cudaStream_t s);
 
 // The whole recursion in the registers of thread-block clusters (cluster.cu).
-constexpr int kMaxCluster = 8;
+constexpr int kMaxCluster = 16;  // above 8 it takes CTAs that fill their SMs and a GPC of that many
 constexpr int kClusterSmem = 226 * 1024;  // dynamic shared memory a CTA may ask for
 constexpr int kClusterBatch = 16;         // steps between two folds of the column sums
 struct ClusterArgs {
@@ -166,9 +166,10 @@ struct ClusterArgs {
 };
 struct ClusterPlan {
   int by, cluster, rows, threads;
+  int rag;  // how the tiles cover the lattice (cluster.cuh)
   size_t smem;
 };
-bool plan_cluster(int Lx, int Ly, int ncols, ClusterPlan *p);
+bool plan_cluster(int Lx, int Ly, int px, int py, int ncols, ClusterPlan *p);
 cudaError_t launch_cluster(ClusterArgs a, const ClusterPlan &p, cudaStream_t s);
 
 // Recursion step for the general lattice (complex vectors; nnn: 8 hopping

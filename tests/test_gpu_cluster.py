@@ -1,6 +1,6 @@
 """The register-resident recursion of thread-block clusters (FP32 real on-site
 lattices with one hopping): moments and order parameter against the FP64
-oracle at the edges of its tiles (4 sites wide, 4, 6 or 8 high), of its CTAs
+oracle at the edges of its tiles (4 sites wide, 4, 6, 8 or 10 high), of its CTAs
 and of its clusters, for every kind of edge, few and many start sites; the
 lattices it does not take (hoppings that differ) against the streamed kernels.
 Tolerances are those of the FP32 recursion: its column sums carry at most
@@ -29,7 +29,7 @@ def lattice(Lx, Ly, px, py, M, seed):
 
 @pytest.mark.parametrize("px,py", [(0, 0), (1, 0), (0, 1), (1, 1)])
 @pytest.mark.parametrize("shape", [(3, 3, 2), (4, 8, 3), (5, 9, 37), (33, 49, 68), (65, 66, 35), (97, 95, 34),
-                                   (130, 127, 36), (256, 250, 20)])
+                                   (130, 127, 36), (256, 250, 20), (500, 319, 21)])
 def test_moments_match_oracle(shape, px, py):
     Lx, Ly, M = shape
     p = lattice(Lx, Ly, px, py, M, seed=Lx * 13 + Ly)
