@@ -59,8 +59,9 @@ bool plan_cluster(int Lx, int Ly, int px, int py, int ncols, ClusterPlan *p) {
     const long long rounds = (ncols + slots - 1) / slots;
     const int busy = static_cast<int>(std::min<long long>(c.per_sm, (ctas + sms - 1) / sms));  // CTAs on an SM
     const double row_cycles = by == 4 ? 31.0 : by == 6 ? 29.3 : by == 8 ? 28.4 : 40.0;
+    const double ragged = c.plan.rag == 2 ? 1.4 : 1.0;  // selects, waits without work in between
     c.cost = static_cast<double>(rounds) * (500.0 + 250.0 * std::log2(static_cast<double>(c.plan.cluster)) +
-                                            row_cycles * ((busy * nw + 3) / 4 * 4) * by);
+                                            ragged * row_cycles * ((busy * nw + 3) / 4 * 4) * by);
   };
   const int TX = (Lx + 3) / 4;
   std::vector<Candidate> list;

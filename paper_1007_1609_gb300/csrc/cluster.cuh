@@ -143,7 +143,8 @@ struct Record {
 };
 
 // RAG 0: the tiles cover the lattice exactly; 1: they stick out over open edges;
-// 2: they stick out over a periodic edge
+// 2: they stick out over a periodic edge (compiled apart: its selects and early
+// waits cost every warp)
 template <int BY, int RAG>
 __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(ClusterArgs a) {
   using Rec = Record<BY>;
@@ -208,6 +209,15 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
   const int w = Lx - kB * (TX - 1);                       // live columns of the last tile of a row
   const bool wrapped = act && rl < BY && a.py;            // periodic y: row rl is the wrapped neighbour row
   const int rsel = (RAG == 2 && tx == TX - 1) ? w - 1 : kB - 1;  // column whose right neighbour is the halo
+
+  // Rows stick out over a periodic y edge: inner rows of the last tiles then need
+  // the row across it, so every warp waits for the end rows first (the last
+  // tiles' warps alone, a step behind the others, measured slower: 25.8 against
+  // 20.1 ms on the 75 x 90 torus).
+  const bool early = RAG == 2 && a.py && Ly % BY != 0;
+  // Warps whose tiles have all their rows (or none) test no row: the map of the
+  // open 75 x 90 lattice 15.4 -> 13.6 ms, of the 500 x 320 slab 48.5 -> 45.1 ms.
+  const bool whole = !early && __all_sync(0xffffffffu, rl == BY || rl == 0);
 
   // where the four neighbour tiles' edges are read
   auto record = [&](int k, int quad) { return e0 + k * Rec::kBytes + quad * 16; };
@@ -347,8 +357,9 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
   // buf_c: the buffer that holds the edges of j_n.  Rows 1 .. BY - 2 first: they
   // need no row of another tile, so their arithmetic (and the warp reduction
   // of the step before) runs while the other warps' end rows are on their way.
-  auto step = [&](int n, int col, auto buf_c, Tile &cu, Tile &cv, Tile &ou, Tile &ov) {
+  auto step = [&](int n, int col, auto buf_c, auto edge_c, Tile &cu, Tile &cv, Tile &ou, Tile &ov) {
     constexpr int rd = decltype(buf_c)::value * Rec::kBuffer, wr = (1 - decltype(buf_c)::value) * Rec::kBuffer;
+    constexpr bool EDGE = decltype(edge_c)::value;  // rows of the tile may be missing
     F2 sa = 0, sb = 0, sc = 0;
     // component part of row r; l, g: the halo left and right, (bl, bh), (tl, th): the halo below row 0 and above row 3
     auto row = [&](int r, int part, const F2 (&er)[2], float l0, float g3, F2 bl, F2 bh, F2 tl, F2 th) {
@@ -387,8 +398,8 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
       er[0] = v.lo;
       er[1] = v.hi;
     };
-    if (RAG == 2) {
-      wait_ends(phase);
+    if (RAG == 2 && EDGE) {
+      if (early) wait_ends(phase);
       if (wrapped) {
         const Quad hu = lds4(up + rd), hv = lds4(up + rd + 16);
 #pragma unroll
@@ -408,7 +419,7 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const int r = 2 * k + 1 + i;
-        if (RAG == 0 || r < rl) {
+        if (!EDGE || r < rl) {
           F2 er[2];
           load_e(r, er);
           row(r, 0, er, el(hl, i), el(hr, i), 0, 0, 0, 0);
@@ -419,7 +430,7 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
     }
     arrive(bar_a);
     reduce(n - 1, A, B, C);
-    if (RAG != 2) wait_ends(phase);
+    if (!(RAG == 2 && EDGE && early)) wait_ends(phase);
     phase ^= 1u;
     // the last batch of sums: reduced by step 1, sent in step 2 and folded in step 3 of the next one
     if (decltype(buf_c)::value == 1 && n % kBatch == 2 && n > 2) send(n - 2);
@@ -429,7 +440,7 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
       const Quad hl = lds4(lf + rd + last), hr = lds4(rt + rd + last);
       {
         const Quad du = lds4(dn + rd), dv = lds4(dn + rd + 16);
-        if (RAG == 0 || 0 < rl) {
+        if (!EDGE || 0 < rl) {
           F2 er[2];
           load_e(0, er);
           row(0, 0, er, el(hl, 0), el(hr, 0), du.lo, du.hi, 0, 0);
@@ -437,7 +448,7 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
         }
       }
       const Quad tu = lds4(up + rd), tv = lds4(up + rd + 16);
-      if (RAG == 0 || BY - 1 < rl) {
+      if (!EDGE || BY - 1 < rl) {
         F2 er[2];
         load_e(BY - 1, er);
         row(BY - 1, 0, er, el(hl, 1), el(hr, 1), 0, 0, tu.lo, tu.hi);
@@ -487,12 +498,16 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
     publish_ends(qu, 0, 0);
     publish_ends(qv, 1, 0);
     arrive_ends();
-    for (int n = 1; n <= a.steps;) {
-      step(n, col, std::integral_constant<int, 0>{}, qu, qv, pu, pv);
-      if (++n > a.steps) break;
-      step(n, col, std::integral_constant<int, 1>{}, pu, pv, qu, qv);
-      ++n;
-    }
+    const auto run = [&](auto edge) {
+      for (int n = 1; n <= a.steps;) {
+        step(n, col, std::integral_constant<int, 0>{}, edge, qu, qv, pu, pv);
+        if (++n > a.steps) break;
+        step(n, col, std::integral_constant<int, 1>{}, edge, pu, pv, qu, qv);
+        ++n;
+      }
+    };
+    if (RAG == 0 || whole) run(std::false_type{});
+    else run(std::true_type{});
     wait(bar_a, phase);
     wait_ends(phase);
     phase ^= 1u;
