@@ -425,6 +425,14 @@ cbdg_status autotune(cbdg_lattice *L, int mode, int n_sites, TuneVal *out) {
   return CBDG_OK;
 }
 
+// Whether the recursions of this lattice may run in the registers of
+// thread-block clusters: real FP32 vectors, one hopping, and no option that asks
+// for a streaming kernel or its tiles.
+bool on_chip(const cbdg_lattice *L) {
+  return mode_of(L) == kReal && L->precision == CBDG_FP32_MIXED && L->uniform && L->resident && L->slab_w == 0 &&
+         L->row_split == 0 && L->depth == 0 && L->temporal == 0 && !L->autotune && !L->stall;
+}
+
 // Runs the recursion for n_sites start vectors (device list), folding the
 // moments into per-column accumulators; optionally writes the moments
 // ([n_sites][M] and [n_sites][M][stride]).  With finalize, Delta_out and n
@@ -457,9 +465,7 @@ cbdg_status run_columns(cbdg_lattice *L, const int32_t *sites, int n_sites, int 
   // real FP32 lattices with one hopping: the whole recursion in the registers
   // of thread-block clusters, one launch
   ClusterPlan plan;
-  if (mode == kReal && L->precision == CBDG_FP32_MIXED && L->uniform && L->resident && L->slab_w == 0 &&
-      L->row_split == 0 && L->depth == 0 && L->temporal == 0 && !L->autotune && !L->stall && n_sites > 0 &&
-      plan_cluster(L->Lx, L->Ly, L->px, L->py, n_sites, &plan)) {
+  if (on_chip(L) && n_sites > 0 && plan_cluster(L->Lx, L->Ly, L->px, L->py, n_sites, &plan)) {
     CK(L->acc_n.ensure(static_cast<size_t>(n_sites) * sizeof(double)));
     CK(L->acc_d.ensure(static_cast<size_t>(n_sites) * 4 * sizeof(double2)));
     ClusterArgs c{};
@@ -1007,6 +1013,56 @@ cbdg_status adjoint_run(cbdg_lattice *L, double T, int M, const int32_t *cols = 
   }
   cbdg_status st = prepare(L, T, CBDG_JACKSON, 0.0, M, map_source);
   if (st != CBDG_OK) return st;
+  // FP32 lattices with one hopping: the whole adjoint in the registers of
+  // thread-block clusters
+  {
+    ClusterPlan plan;
+    int clusters = 0;
+    size_t ck_bytes = 0, acc_bytes = 0;
+    if (on_chip(L) &&
+        plan_adjoint_cluster(L->Lx, L->Ly, L->px, L->py, n_cols, M, &plan, &clusters, &ck_bytes, &acc_bytes) &&
+        (L->ws_mb == 0 || ck_bytes + acc_bytes <= static_cast<size_t>(L->ws_mb) << 20)) {
+      CK(L->adj_ck.ensure(ck_bytes));
+      CK(L->adj_part.ensure(acc_bytes));
+      CK(cudaMemsetAsync(L->adj_part.p, 0, acc_bytes, L->stream));
+      CK(L->adj_out.ensure(static_cast<size_t>(N) * 6 * sizeof(double)));
+      AdjointClusterArgs c{};
+      c.params = L->params.as<float>();
+      c.scal = L->scal.as<double>();
+      c.eps = L->eps.as<double>();
+      c.delta = L->delta.as<double2>();
+      c.sites = cols;
+      c.ck = L->adj_ck.as<float4>();
+      c.acc = L->adj_part.as<float2>();
+      c.flags = L->flags.as<unsigned int>();
+      c.mu = L->mu;
+      c.hop = L->hop_all;
+      c.Lx = L->Lx;
+      c.Ly = L->Ly;
+      c.px = L->px;
+      c.py = L->py;
+      c.ncols = n_cols;
+      c.M = M;
+      if (map_source) {
+        // y_m = w_i (U_i / 2) C_m on the hole row
+        c.w = L->adj_w.as<double>();
+        c.u = L->coupling_site();
+        c.tab = L->C.as<double>();
+        c.scale = L->site_cpl ? 0.5 : 0.5 * L->coupling;
+        c.part = 1;
+      } else {
+        // y_m = src[c][m] on the electron row
+        c.tab = src;
+        c.stride = M;
+        c.scale = 1.0;
+      }
+      CK(launch_adjoint_cluster(c, plan, clusters, L->stream));
+      double *ge = L->adj_out.as<double>(), *gd = ge + N, *gh = ge + 2 * N;
+      CK(launch_adjoint_cluster_final(c, plan, clusters, ge, gh, gd, L->stream));
+      L->launches += 2;
+      return CBDG_OK;
+    }
+  }
   std::vector<double> hC(M);
   CK(cudaMemcpyAsync(hC.data(), L->C.p, M * sizeof(double), cudaMemcpyDeviceToHost, L->stream));
   CK(cudaStreamSynchronize(L->stream));

@@ -172,6 +172,31 @@ struct ClusterPlan {
 bool plan_cluster(int Lx, int Ly, int px, int py, int ncols, ClusterPlan *p);
 cudaError_t launch_cluster(ClusterArgs a, const ClusterPlan &p, cudaStream_t s);
 
+// The adjoint of adjoint.cu in the registers of thread-block clusters
+// (adjoint_cluster.cuh): sources as in PassSource, with the column's table at
+// tab + stride * column.
+struct AdjointClusterArgs {
+  const float *params;     // [N][kParamStride]
+  const double *scal, *eps;
+  const double2 *delta;
+  const int32_t *sites;    // [ncols]
+  const double *w, *u, *tab;
+  float4 *ck;              // [CTAs][n_ck][16][threads] kept pairs
+  float2 *acc;             // [CTAs][64][threads] gradient sums, zero before the first launch
+  unsigned int *flags;
+  double mu, hop, scale;
+  int stride, part, n_ck;
+  int Lx, Ly, px, py, ncols, M;
+  int cluster, rows;
+};
+// Plans the launch for ncols columns and M moments; false where the lattice or M
+// does not fit.  clusters: how many run; ck_bytes and acc_bytes: their scratch.
+bool plan_adjoint_cluster(int Lx, int Ly, int px, int py, int ncols, int M, ClusterPlan *p, int *clusters,
+                          size_t *ck_bytes, size_t *acc_bytes);
+cudaError_t launch_adjoint_cluster(AdjointClusterArgs a, const ClusterPlan &p, int clusters, cudaStream_t s);
+cudaError_t launch_adjoint_cluster_final(const AdjointClusterArgs &a, const ClusterPlan &p, int clusters, double *g_eps,
+                                         double *g_hop, double *g_delta, cudaStream_t s);
+
 // Recursion step for the general lattice (complex vectors; nnn: 8 hopping
 // directions; bond: nearest-neighbour pairing, which skips the column sums).
 // The partial sums, when formed, are [row_split][4][ld].

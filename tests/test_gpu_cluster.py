@@ -99,3 +99,39 @@ def test_ensemble_mixes_both_kernels():
         ref, _, _, _ = orc.scf(as_oracle(p), 0.02, 48, K, 0.5, 0.0, 2)
         assert max_abs(ens.delta(k), ref) < TOL["fp32"][1]
     ens.close()
+
+
+@pytest.mark.parametrize("shape", [(3, 2, 0, 0, 2), (4, 4, 1, 1, 3), (9, 7, 0, 0, 10), (12, 8, 1, 0, 11),
+                                   (33, 30, 0, 0, 20), (8, 36, 0, 1, 67), (66, 70, 0, 0, 66), (130, 67, 0, 0, 12)])
+def test_backward_matches_oracle(shape):
+    """The adjoint in cluster registers: every remainder of its kept pairs (8
+    steps) and of its sums (64), one CTA and clusters, tiles that stick out,
+    periodic sides.  Against the oracle's reverse mode within the FP32
+    gradient tolerance (1e-3 of the largest component), and against the
+    streamed adjoint within 2e-5 (both carry the rounding of M FP32 steps)."""
+    Lx, Ly, px, py, M = shape
+    p = lattice(Lx, Ly, px, py, M, seed=Lx + M)
+    w = np.random.default_rng(M).normal(size=p.N)
+    lat = gpu_lattice(p, "fp32")
+    cbdg.cbdg_launch_count(lat.handle, reset=True)
+    got = lat.backward(p.T, M, w.astype(np.complex128))
+    assert cbdg.cbdg_launch_count(lat.handle) < 12  # one recursion launch, not one per step
+    ref = gpu_lattice(p, "fp32", resident=0).backward(p.T, M, w.astype(np.complex128))
+    for x, y in zip(got, ref):
+        assert max_abs(x, y) <= 2e-5 * max(np.max(np.abs(y)), 1e-3)
+    if p.N <= 1000:
+        o = orc.scf_map_gradient(as_oracle(p), lat.rescale, orc.fold_coefficients(M, K, lat.rescale, p.T), w)
+        for x, y in zip(got, o):
+            assert max_abs(x.real.reshape(-1), np.asarray(y).reshape(-1)) <= 1e-3 * max(np.max(np.abs(y)), 1e-6)
+
+
+def test_ldos_backward_matches_streamed():
+    """The LDOS loss's source (the electron rows, a table per column) through
+    the adjoint in cluster registers against the streamed one."""
+    p = lattice(28, 20, 0, 0, 90, seed=12)
+    lat, ref = gpu_lattice(p, "fp32"), gpu_lattice(p, "fp32", resident=0)
+    sites = np.array([0, 27, 300, 559, 300], dtype=np.int32)
+    E = np.linspace(-2.0, 2.0, 9)
+    G = np.random.default_rng(4).normal(size=(5, 9))
+    for x, y in zip(lat.ldos_backward(sites, 90, E, G), ref.ldos_backward(sites, 90, E, G)):
+        assert max_abs(x, y) <= 2e-5 * np.max(np.abs(y))
