@@ -426,11 +426,76 @@ cbdg_status autotune(cbdg_lattice *L, int mode, int n_sites, TuneVal *out) {
 }
 
 // Whether the recursions of this lattice may run in the registers of
-// thread-block clusters: real FP32 vectors, one hopping, and no option that asks
-// for a streaming kernel or its tiles.
-bool on_chip(const cbdg_lattice *L) {
-  return mode_of(L) == kReal && L->precision == CBDG_FP32_MIXED && L->uniform && L->resident && L->slab_w == 0 &&
-         L->row_split == 0 && L->depth == 0 && L->temporal == 0 && !L->autotune && !L->stall;
+// thread-block clusters: FP32 vectors and no option that asks for a streaming
+// kernel or its tiles; real ones with one hopping in cluster.cuh's form.
+bool on_chip_options(const cbdg_lattice *L) {
+  return L->precision == CBDG_FP32_MIXED && L->resident && L->slab_w == 0 && L->row_split == 0 && L->depth == 0 &&
+         L->temporal == 0 && !L->autotune && !L->stall;
+}
+bool on_chip(const cbdg_lattice *L) { return mode_of(L) == kReal && L->uniform && on_chip_options(L); }
+
+// Adds the device time of one on-chip recursion launch to the profile (it moves no vectors).
+cbdg_status profile_one(cbdg_lattice *L, cudaEvent_t e0, cudaEvent_t e1) {
+  CK(cudaEventSynchronize(e1));
+  float ms = 0.f;
+  CK(cudaEventElapsedTime(&ms, e0, e1));
+  L->prof_ms += ms;
+  L->prof_launches += 1;
+  return CBDG_OK;
+}
+cbdg_status two_events(cbdg_lattice *L) {
+  while (L->events.size() < 2) {
+    cudaEvent_t ev;
+    CK(cudaEventCreate(&ev));
+    L->events.push_back(ev);
+  }
+  return CBDG_OK;
+}
+
+// The direct recursion of a general FP32 lattice on chip: c holds what is read
+// of each moment.  *ran: whether the lattice fits.
+cbdg_status run_cplx_on_chip(cbdg_lattice *L, const void *params, const int32_t *sites, int n_sites, int M, double tol,
+                             CplxClusterArgs c, bool *ran) {
+  ClusterPlan plan;
+  int clusters = 0;
+  const int bond = L->pairing == CBDG_BOND_V ? 1 : 0;
+  *ran = false;
+  if (!on_chip_options(L) || n_sites < 1 ||
+      !plan_cluster_cplx(L->Lx, L->Ly, L->px, L->py, L->n_dirs == 8, bond, n_sites, &plan, &clusters))
+    return CBDG_OK;
+  c.params = static_cast<const float *>(params);
+  c.scal = L->scal.as<double>();
+  c.C = L->C.as<double>();
+  c.eps = L->eps.as<double>();
+  c.hop = L->hop.as<double2>();
+  c.delta = L->delta.as<double2>();
+  c.sites = sites;
+  c.flags = L->flags.as<unsigned int>();
+  c.mu = L->mu;
+  c.tol = tol;
+  c.n_dirs = L->n_dirs;
+  c.Lx = L->Lx;
+  c.Ly = L->Ly;
+  c.px = L->px;
+  c.py = L->py;
+  c.ncols = n_sites;
+  c.M = M;
+  if (L->profile) {
+    const cbdg_status st = two_events(L);
+    if (st != CBDG_OK) return st;
+    CK(cudaEventRecord(L->events[0], L->stream));
+  }
+  CK(launch_cluster_cplx(c, bond, plan, clusters, L->stream));
+  L->launches += 1;
+  if (L->profile) {
+    CK(cudaEventRecord(L->events[1], L->stream));
+    const cbdg_status st = profile_one(L, L->events[0], L->events[1]);
+    if (st != CBDG_OK) return st;
+  }
+  L->last_cfg = StepConfig{2, 0, 1, plan.threads, 0};  // depth 0: on chip
+  L->last_temporal = 1;
+  *ran = true;
+  return CBDG_OK;
 }
 
 // Runs the recursion for n_sites start vectors (device list), folding the
@@ -491,8 +556,18 @@ cbdg_status run_columns(cbdg_lattice *L, const int32_t *sites, int n_sites, int 
     c.M = M;
     c.steps = (M + 1) / 2 - 1;
     c.mom_stride = mom_stride;
+    if (L->profile) {
+      const cbdg_status st = two_events(L);
+      if (st != CBDG_OK) return st;
+      CK(cudaEventRecord(L->events[0], L->stream));
+    }
     CK(launch_cluster(c, plan, L->stream));
     L->launches += 1;
+    if (L->profile) {
+      CK(cudaEventRecord(L->events[1], L->stream));
+      const cbdg_status st = profile_one(L, L->events[0], L->events[1]);
+      if (st != CBDG_OK) return st;
+    }
     if (finalize) {
       CK(launch_finalize_onsite(n_sites, sites, L->coupling, L->coupling_site(), L->acc_n.as<double>(),
                                 L->acc_d.as<double2>(), L->dout.as<double2>(), L->nout.as<double>(), L->stream));
@@ -501,6 +576,35 @@ cbdg_status run_columns(cbdg_lattice *L, const int32_t *sites, int n_sites, int 
     L->last_cfg = StepConfig{1, 0, 1, plan.threads, 0};  // depth 0: on chip
     L->last_temporal = 1;
     return CBDG_OK;
+  }
+  // bond pairing, FP32: the direct recursion on chip
+  if (mode == kDirect) {
+    double *accn = nullptr;
+    double2 *accb = nullptr;
+    if (finalize) {
+      CK(L->acc_site_n.ensure(static_cast<size_t>(L->N) * sizeof(double)));
+      CK(L->acc_site_b.ensure(static_cast<size_t>(L->N) * 4 * sizeof(double2)));
+      accn = L->acc_site_n.as<double>();
+      accb = L->acc_site_b.as<double2>();
+      CK(cudaMemsetAsync(accn, 0, static_cast<size_t>(n_sites) * sizeof(double), L->stream));
+      CK(cudaMemsetAsync(accb, 0, static_cast<size_t>(n_sites) * 4 * sizeof(double2), L->stream));
+    }
+    CplxClusterArgs c{};
+    c.mode = kReadBonds;
+    c.n_t = 5;
+    c.acc_n = accn;
+    c.acc = accb;
+    c.a_re = mom_ee;
+    c.a_h = mom_eh;
+    bool ran = false;
+    const cbdg_status st = run_cplx_on_chip(L, L->params.p, sites, n_sites, M, 1e-4, c, &ran);
+    if (st != CBDG_OK) return st;
+    if (ran && finalize) {
+      CK(launch_finalize_bond(L->N, L->Lx, L->Ly, L->px, L->py, L->coupling, L->coupling_site(), accn, accb,
+                              L->dout.as<double2>(), L->nout.as<double>(), L->stream));
+      L->launches += 1;
+    }
+    if (ran) return CBDG_OK;
   }
   // small real lattices: the whole recursion in shared memory, one launch
   const int Wres = (mode == kReal && L->resident && L->slab_w == 0 && L->row_split == 0 && L->depth == 0 &&
@@ -847,6 +951,18 @@ cbdg_status run_targets(cbdg_lattice *L, const int32_t *sites, int n_sites, int 
                           L->params_c.p, L->stream));
     L->launches += 1;
     params = L->params_c.p;
+  }
+  if (!acc || n_t <= 8) {
+    CplxClusterArgs c{};
+    c.mode = kReadTargets;
+    c.n_t = n_t;
+    c.targets = targets;
+    c.acc = acc;
+    c.a_e = a_e;
+    c.a_h = a_h;
+    bool ran = false;
+    const cbdg_status st = run_cplx_on_chip(L, params, sites, n_sites, M, 1e-4, c, &ran);
+    if (st != CBDG_OK || ran) return st;
   }
   const size_t es = 2 * elem_size(L);
   const size_t rows = 2 * static_cast<size_t>(L->N);

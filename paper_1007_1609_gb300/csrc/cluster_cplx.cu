@@ -1,0 +1,93 @@
+// cluster_cplx.cu -- plan and dispatch of the register-resident recursion of
+// general lattices (cluster_cplx.cuh).
+#include <algorithm>
+#include <cmath>
+#include <map>
+#include <mutex>
+#include <tuple>
+
+#include "internal.h"
+
+namespace cbdg {
+
+#define CBDG_CPLX(nnn, bond)                                                                                     \
+  int cplx_slots_##nnn##_##bond(const ClusterPlan &p);                                                           \
+  cudaError_t cplx_launch_##nnn##_##bond(const CplxClusterArgs &a, const ClusterPlan &p, int clusters, cudaStream_t s);
+CBDG_CPLX(0, 0)
+CBDG_CPLX(0, 1)
+CBDG_CPLX(1, 0)
+CBDG_CPLX(1, 1)
+#undef CBDG_CPLX
+
+namespace {
+
+constexpr int kRecord = 33, kCols = 2, kMaxThreads = 384;  // as in cluster_cplx.cuh
+
+// p.rag: nnn + 2 bond
+int slots_of(const ClusterPlan &p) {
+  static std::mutex mutex;
+  static std::map<std::tuple<int, int, int, int, size_t>, int> known;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lock(mutex);
+  const auto key = std::make_tuple(dev, p.rag, p.cluster, p.threads, p.smem);
+  const auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  const int n = p.rag == 0   ? cplx_slots_0_0(p)
+                : p.rag == 1 ? cplx_slots_1_0(p)
+                : p.rag == 2 ? cplx_slots_0_1(p)
+                             : cplx_slots_1_1(p);
+  return known[key] = n;
+}
+
+}  // namespace
+
+// Cycles of a step of all columns, by clusters: a round takes 900 for the chain through shared
+// memory, 250 for each doubling of the cluster (its barrier) and the shared-memory wavefronts of
+// the warps on an SM; fitted to 32 .. 800 columns of 16 x 16 .. 140 x 120 sites, within 15 %.
+// Falls short (false) where the streamed kernels are expected to be faster.
+bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int ncols, ClusterPlan *p, int *clusters) {
+  if ((px && Lx % 4) || (py && Ly % 2) || ncols < 1) return false;
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int TX = (Lx + 3) / 4, TY = (Ly + 1) / 2, pairs = (ncols + kCols - 1) / kCols;
+  const double warp_cycles = nnn ? (bond ? 355.0 : 285.0) : (bond ? 255.0 : 215.0);
+  double best = 0.0;
+  for (int cluster = 1; cluster <= kMaxCluster && cluster <= TY; ++cluster) {
+    const int rows = (TY + cluster - 1) / cluster, threads = (TX * rows + 31) / 32 * 32 * kCols;
+    if ((TY + rows - 1) / rows != cluster || threads > kMaxThreads) continue;
+    ClusterPlan q{2, cluster, rows, threads, nnn + 2 * bond,
+                  static_cast<size_t>(TX * rows + (cluster > 1 ? TX : 0) + 1) * 2 * kRecord * 16};
+    if (q.smem > kCplxClusterSmem) continue;
+    const int slots = slots_of(q);
+    if (slots < 1) continue;
+    const int nw = threads / 32;
+    const int per_sm = std::max(1, std::min(12 / nw, static_cast<int>(kClusterSmem / (q.smem + 4096))));
+    const long long rounds = (pairs + slots - 1) / slots, ctas = static_cast<long long>(pairs) * cluster;
+    const int busy = static_cast<int>(std::min<long long>(per_sm, (ctas + sms - 1) / sms));
+    const double cost = static_cast<double>(rounds) *
+                        (900.0 + 250.0 * std::log2(static_cast<double>(cluster)) + warp_cycles * busy * nw);
+    if (best == 0.0 || cost < best) {
+      best = cost;
+      *p = q;
+      *clusters = std::min(slots, pairs);
+    }
+  }
+  // The streamed kernels take 21,000 cycles a step (launches, latency) and 0.0165 a site and
+  // vector.  Streamed -> on chip, ms, eight hoppings and bond pairing, M = 400: 40 x 36,
+  // 400 columns: 6.0 -> 2.3; 64 x 64: 9.3 -> 5.5; 96 x 96: 18.3 -> 9.8; 1000 columns:
+  // 41.8 -> 28.3; 120 x 120: 57.2 -> 48.5; 100 x 98: 45.0 -> 42.2.  Clusters of 13 to 16 CTAs
+  // fit the chip only seven times (112 of the 152 SMs), and many columns of them stay
+  // streamed (128 x 128, 800 columns, M = 200: 31.7 ms, 33.4 on chip).
+  return best > 0.0 && best < 21000.0 + 0.0165 * Lx * Ly * ncols;
+}
+
+cudaError_t launch_cluster_cplx(CplxClusterArgs a, int bond, const ClusterPlan &p, int clusters, cudaStream_t s) {
+  a.cluster = p.cluster;
+  a.rows = p.rows;
+  if (bond) return p.rag & 1 ? cplx_launch_1_1(a, p, clusters, s) : cplx_launch_0_1(a, p, clusters, s);
+  return p.rag & 1 ? cplx_launch_1_0(a, p, clusters, s) : cplx_launch_0_0(a, p, clusters, s);
+}
+
+}  // namespace cbdg

@@ -1,0 +1,11 @@
+// The register-resident recursion of general lattices (cluster_cplx.cuh): nearest neighbours, on-site pairing.
+#include "cluster_cplx.cuh"
+
+namespace cbdg {
+
+int cplx_slots_0_0(const ClusterPlan &p) { return cplx_slots_one<false, false>(p); }
+cudaError_t cplx_launch_0_0(const CplxClusterArgs &a, const ClusterPlan &p, int clusters, cudaStream_t s) {
+  return cplx_launch_one<false, false>(a, p, clusters, s);
+}
+
+}  // namespace cbdg

@@ -197,6 +197,33 @@ cudaError_t launch_adjoint_cluster(AdjointClusterArgs a, const ClusterPlan &p, i
 cudaError_t launch_adjoint_cluster_final(const AdjointClusterArgs &a, const ClusterPlan &p, int clusters, double *g_eps,
                                          double *g_hop, double *g_delta, cudaStream_t s);
 
+// The direct recursion of general lattices (FP32) in the registers of
+// thread-block clusters (cluster_cplx.cuh), and what is read of every j_m:
+//   kReadBonds:   <e_i|j_m> (real part a_re [ncols][M]), <h_i|j_m> and the four
+//                 <h_{i+d}|j_m> (a_h [ncols][M][5]); acc_n -= sum C_m Re<e_i|j_m>,
+//                 acc[col][d] += sum C_m conj<h_{i+d}|j_m>;  n_t = 5
+//   kReadTargets: <e_t|j_m>, <h_t|j_m> (a_e, a_h [ncols][M][n_t]) at n_t targets, or
+//                 at the neighbours along directions 0 .. n_t - 1 (targets null),
+//                 acc[col][t] += sum C_m <e_t|j_m> (n_t <= 8)
+// Any output may be null.
+enum { kReadBonds = 0, kReadTargets = 1 };
+struct CplxClusterArgs {
+  const float *params;     // as for step_cplx.cu
+  const double *scal, *C, *eps;
+  const double2 *hop, *delta;
+  const int32_t *sites, *targets;
+  double *acc_n, *a_re;
+  double2 *acc, *a_e, *a_h;
+  unsigned int *flags;
+  double mu, tol;
+  int mode, n_t, n_dirs;
+  int Lx, Ly, px, py, ncols, M;
+  int cluster, rows;
+};
+constexpr int kCplxClusterSmem = 227 * 1024 - 3104;  // dynamic shared memory beside the kernel's own
+bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int ncols, ClusterPlan *p, int *clusters);
+cudaError_t launch_cluster_cplx(CplxClusterArgs a, int bond, const ClusterPlan &p, int clusters, cudaStream_t s);
+
 // Recursion step for the general lattice (complex vectors; nnn: 8 hopping
 // directions; bond: nearest-neighbour pairing, which skips the column sums).
 // The partial sums, when formed, are [row_split][4][ld].
