@@ -120,7 +120,7 @@ struct cbdg_lattice {
   DBuf vec2, vec3;  // the out-of-place outputs of the row-block passes
   DBuf acc_site_n, acc_site_b, adj_ck, adj_seg, adj_lam, adj_part, adj_w, adj_out, adj_fp;
   DBuf adj_wc, adj_outc;  // general-lattice adjoint: dL/dDelta_out (complex) and the gradients
-  DBuf params_c, g_acc, g_tgt, g_mom, g_w, g_out;  // nonlocal readout (green.cu)
+  DBuf params_c, g_acc, g_tgt, g_mom, g_w, g_out, g_dig;  // nonlocal readout (green.cu)
   DBuf cpl;              // coupling per Delta entry (cbdg_set_coupling)
   DBuf sym_rep, sym_list;  // cbdg_set_symmetry: representative of every site, distinct representatives
   int sym_n = 0;           // number of representatives (0: no symmetry reduction)
@@ -1754,7 +1754,7 @@ cbdg_status cbdg_destroy(cbdg_lattice *L) {
                   &L->f,       &L->C,     &L->sites_all, &L->sites_user, &L->vec0, &L->vec1,
                   &L->partials, &L->mu1,  &L->dA,    &L->acc_n,   &L->acc_d, &L->dout,
                   &L->nout,    &L->mom_ee, &L->mom_eh, &L->stage, &L->acc_site_n, &L->acc_site_b, &L->adj_ck, &L->adj_seg, &L->adj_lam, &L->adj_part, &L->adj_w, &L->adj_out, &L->adj_fp,
-                  &L->params_c, &L->g_acc, &L->g_tgt, &L->g_mom, &L->g_w, &L->g_out, &L->cpl};
+                  &L->params_c, &L->g_acc, &L->g_tgt, &L->g_mom, &L->g_w, &L->g_out, &L->g_dig, &L->cpl};
   for (DBuf *b : bufs) b->release();
   for (cudaEvent_t ev : L->events) cudaEventDestroy(ev);
   L->drop_graph();
@@ -2004,13 +2004,24 @@ cbdg_status cbdg_green_function(cbdg_lattice *L, const int32_t *sites, int32_t n
   CK(cudaMemcpyAsync(dE, he.data(), e_bytes, cudaMemcpyHostToDevice, L->stream));
   CK(launch_green_weights(n_E, M, kernel, lambda, dE, L->scal.as<double>(), W, L->stream));
   L->launches += 1;
+  // on the tensor cores, where the digit planes (half a gigabyte at most) fit the device
+  const long long rows = static_cast<long long>(n_sites) * n_targets;
+  bool digits = green_mma_wanted(rows, M, n_E);
+  if (digits) {
+    const cudaError_t ge = L->g_dig.ensure(green_mma_scratch(rows, M, n_E));
+    if (ge == cudaErrorMemoryAllocation) cudaGetLastError();
+    else CK(ge);
+    digits = ge == cudaSuccess;
+  }
   cbdg_complex *outs[2] = {G11, G12};
   const double2 *moms[2] = {me, mh};
   for (int p = 0; p < 2; ++p) {
     if (!outs[p]) continue;
     double2 *dst = is_device_ptr(outs[p]) ? reinterpret_cast<double2 *>(outs[p]) : gbuf[p];
-    CK(launch_green_contract(n_sites, n_targets, M, n_E, moms[p], W, dst, L->stream));
-    L->launches += 1;
+    int n = 1;
+    if (digits) CK(launch_green_mma(n_sites, n_targets, M, n_E, moms[p], W, dst, L->g_dig.p, &n, L->stream));
+    else CK(launch_green_contract(n_sites, n_targets, M, n_E, moms[p], W, dst, L->stream));
+    L->launches += n;
     if (dst != reinterpret_cast<double2 *>(outs[p])) CK(deliver(L, outs[p], dst, g_bytes));
   }
   CK(cudaStreamSynchronize(L->stream));  // he is read by the copy above

@@ -104,7 +104,9 @@ __global__ void green_weights_kernel(int n_E, int M, int kernel, double lambda,
 // G[(c*n_t + t)*n_E + e] = sum_n mom[(c*M + n)*n_t + t] W[e][n]  (complex).
 // A CTA owns 16 targets x 64 energies of one start site; each thread keeps
 // four energies of one target and the moment chunks of 32 pass through
-// shared memory.
+// shared memory.  For short sums (M < 64) and where the digit planes of
+// green_mma.cu do not fit: 64 x 64 outputs take 39 us at M = 32 (42 there) and 75 at
+// M = 64 (43).
 constexpr int kGT = 16, kGE = 64, kGN = 32;
 
 __global__ void __launch_bounds__(256) green_contract_kernel(int n_sites, int n_t, int M, int n_E,

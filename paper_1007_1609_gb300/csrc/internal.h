@@ -273,6 +273,11 @@ cudaError_t launch_green_weights(int n_E, int M, int kernel, double lambda, cons
                                  const double *scal, double2 *W, cudaStream_t s);
 cudaError_t launch_green_contract(int n_sites, int n_t, int M, int n_E, const double2 *mom,
                                   const double2 *W, double2 *G, cudaStream_t s);
+// The same contraction on the tensor cores (green_mma.cu), with scratch for its digit planes.
+bool green_mma_wanted(long long rows, int M, int n_E);
+size_t green_mma_scratch(long long rows, int M, int n_E);
+cudaError_t launch_green_mma(int n_sites, int n_t, int M, int n_E, const double2 *mom, const double2 *W, double2 *G,
+                             void *scratch, int *launches, cudaStream_t s);
 
 // ---- auxiliary kernels (aux.cu) -------------------------------------------
 cudaError_t launch_gershgorin(int N, int n_dirs, int pairing, int Lx, int Ly, int px, int py,
