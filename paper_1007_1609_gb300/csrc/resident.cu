@@ -17,7 +17,10 @@
 // every kCheckEvery steps and at the last step for the |mu| <= 1 check (the
 // norm of j_n grows monotonically once a is too small); on GB300, where FP64
 // runs at 1/64 of the FP32 rate, the shuffle tree of every step would cost as
-// much as the stencil.  FP32 without moment output folds linearly too, its
+// much as the stencil.  The shares take one multiply-add a sum, of weights -2 C
+// made once: formed at each use they took nine of the 27 FP64 operations of a thread
+// with one site (16 x 16, M = 256: 534 us an iteration, 497 with them in the table).
+// FP32 without moment output folds linearly too, its
 // per-thread shares in compensated FP32 (the coefficients' FP32 copy times
 // the FP32 partial sums), so that no single folding thread sits on the
 // critical path of every step.  No vector traffic reaches HBM; for the 16 x 16
@@ -42,14 +45,14 @@ struct alignas(sizeof(S) * VEC) Pack {
 template <typename S>
 struct LinAcc {
   double s = 0.0;
-  __device__ __forceinline__ void add(double x) { s += x; }
+  __device__ __forceinline__ void add(double w, double x) { s = fma(w, x, s); }
   __device__ __forceinline__ double value() const { return s; }
 };
 template <>
 struct LinAcc<float> {
   float s = 0.f, c = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    const float y = __fsub_rn(x, c);
+  __device__ __forceinline__ void add(float w, float x) {
+    const float y = __fsub_rn(__fmul_rn(w, x), c);
     const float t = __fadd_rn(s, y);
     c = __fsub_rn(__fsub_rn(t, s), y);
     s = t;
@@ -90,7 +93,7 @@ __global__ void __launch_bounds__(kThreads) resident_kernel(ResidentArgs a) {
   S *bp = reinterpret_cast<S *>(wred + 2 * kWarps * 3 * W);                // j_{n-1} -> j_{n+1}
   S *bq = bp + slab_el;                                                    // j_n
   S *par = bq + slab_el;                                                   // [N][kParamStride]
-  S *Cf = par + static_cast<size_t>(N) * kParamStride;                     // [M] C in S precision
+  S *Cf = par + static_cast<size_t>(N) * kParamStride;                     // [M] -2 C in S precision
 
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int q = t % QUADS, ts = t / QUADS;
@@ -106,7 +109,7 @@ __global__ void __launch_bounds__(kThreads) resident_kernel(ResidentArgs a) {
     for (size_t k = t; k < static_cast<size_t>(N) * kParamStride; k += kThreads) par[k] = gp[k];
     for (int k = t; k < M; k += kThreads) {
       Cs[k] = a.C[k];
-      Cf[k] = static_cast<S>(a.C[k]);
+      Cf[k] = S(-2) * static_cast<S>(a.C[k]);
     }
   }
   // the fold state of column t (threads t < W)
@@ -167,10 +170,10 @@ __global__ void __launch_bounds__(kThreads) resident_kernel(ResidentArgs a) {
     if (LINEAR) {
 #pragma unroll
       for (int l = 0; l < VEC; ++l) {
-        if (m0 < M) ln[l].add(S(-2) * Cf[m0] * pa[l]);
+        if (m0 < M) ln[l].add(Cf[m0], pa[l]);
         if (mo < M) {
-          ln[l].add(S(-2) * Cf[mo] * pb[l]);
-          ld_[l].add(((n & 1) ? S(2) : S(-2)) * Cf[mo] * pc[l]);
+          ln[l].add(Cf[mo], pb[l]);
+          ld_[l].add((n & 1) ? -Cf[mo] : Cf[mo], pc[l]);
         }
       }
     }
