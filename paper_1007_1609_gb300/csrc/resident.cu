@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kThreads) resident_kernel(ResidentArgs a) {
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double *Cs = reinterpret_cast<double *>(smem_raw);                       // [M]
-  double *wred = Cs + M;                                                   // [2][kWarps][3][W]
+  double *wred = Cs + ((M + 1) & ~1);                                      // [2][kWarps][3][W] (slabs: 16-byte rows)
   S *bp = reinterpret_cast<S *>(wred + 2 * kWarps * 3 * W);                // j_{n-1} -> j_{n+1}
   S *bq = bp + slab_el;                                                    // j_n
   S *par = bq + slab_el;                                                   // [N][kParamStride]
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(kThreads) resident_kernel(ResidentArgs a) {
 
 template <typename S, int W>
 size_t smem_bytes(int N, int M) {
-  return static_cast<size_t>(M) * 8 + static_cast<size_t>(2) * kWarps * 3 * W * 8 +
+  return static_cast<size_t>((M + 1) & ~1) * 8 + static_cast<size_t>(2) * kWarps * 3 * W * 8 +
          (static_cast<size_t>(4) * N * W + static_cast<size_t>(N) * kParamStride + M) * sizeof(S);
 }
 
