@@ -607,10 +607,15 @@ cbdg_status run_columns(cbdg_lattice *L, const int32_t *sites, int n_sites, int 
     if (ran) return CBDG_OK;
   }
   // small real lattices: the whole recursion in shared memory, one launch
-  const int Wres = (mode == kReal && L->resident && L->slab_w == 0 && L->row_split == 0 && L->depth == 0 &&
+  int Wres = (mode == kReal && L->resident && L->slab_w == 0 && L->row_split == 0 && L->depth == 0 &&
                     !L->autotune && !L->stall)
                        ? plan_resident(L->precision, L->Lx, L->Ly, n_sites, M)
                        : 0;
+  // .. in FP64 with one hopping, in a form of fewer operations and less memory
+  const bool res_uniform = mode == kReal && L->precision != CBDG_FP32_MIXED && L->uniform && L->resident &&
+                           L->slab_w == 0 && L->row_split == 0 && L->depth == 0 && L->temporal == 0 && !L->autotune &&
+                           !L->stall && plan_resident_uniform(L->Lx, L->Ly, L->px, L->py, n_sites, M, Wres);
+  if (res_uniform) Wres = 1;
   if (Wres) W = Wres;
   int tuned_k = 0, tuned_dm = 0;
   if (!Wres && L->autotune && L->slab_w == 0 && L->row_split == 0 && L->depth == 0 && n_sites > 0) {
@@ -672,10 +677,16 @@ cbdg_status run_columns(cbdg_lattice *L, const int32_t *sites, int n_sites, int 
                           L->scal.as<double>(), L->C.as<double>(), M, L->vec0.p, L->vec1.p,
                           L->mu1.as<double>(), L->dA.as<double2>(), L->acc_n.as<double>(),
                           L->acc_d.as<double2>(), mee, meh, mom_stride, L->stream));
-      CK(launch_resident(L->precision, W, L->Lx, L->Ly, ld, ncols, M, (M + 1) / 2 - 1, L->vec0.p, L->vec1.p,
-                         L->params.p, L->C.as<double>(), L->mu1.as<double>(), L->dA.as<double2>(),
-                         L->acc_n.as<double>(), L->acc_d.as<double2>(), mee, meh, mom_stride,
-                         L->flags.as<unsigned int>(), tol, L->stream));
+      if (res_uniform)
+        CK(launch_resident_uniform(L->Lx, L->Ly, L->px, L->py, ncols, M, (M + 1) / 2 - 1, L->hop_all, L->vec0.p,
+                                   L->vec1.p, L->params.p, L->scal.as<double>(), L->C.as<double>(), L->mu1.as<double>(),
+                                   L->dA.as<double2>(), L->acc_n.as<double>(), L->acc_d.as<double2>(), mee, meh,
+                                   mom_stride, L->flags.as<unsigned int>(), tol, L->stream));
+      else
+        CK(launch_resident(L->precision, W, L->Lx, L->Ly, ld, ncols, M, (M + 1) / 2 - 1, L->vec0.p, L->vec1.p,
+                           L->params.p, L->C.as<double>(), L->mu1.as<double>(), L->dA.as<double2>(),
+                           L->acc_n.as<double>(), L->acc_d.as<double2>(), mee, meh, mom_stride,
+                           L->flags.as<unsigned int>(), tol, L->stream));
       L->launches += 2;
       if (finalize) {
         CK(launch_finalize_onsite(ncols, sites + c0, L->coupling, L->coupling_site(), L->acc_n.as<double>(),

@@ -142,6 +142,15 @@ cudaError_t launch_resident(int precision, int W, int Lx, int Ly, int ld, int nc
                             double *mu_ee, double2 *mu_eh, int mom_stride, unsigned int *flags, double tol,
                             cudaStream_t s);
 
+// The same in FP64 for lattices with one hopping (resident_uniform.cu), at slab width 1.
+// W_general: what plan_resident returned; false where that kernel or the streamed ones are expected to be faster.
+bool plan_resident_uniform(int Lx, int Ly, int px, int py, int ncols, int M, int W_general);
+cudaError_t launch_resident_uniform(int Lx, int Ly, int px, int py, int ncols, int M, int steps, double hop,
+                                    const void *j0, const void *j1, const void *params, const double *scal,
+                                    const double *C, const double *mu1, const double2 *dA, double *acc_n, double2 *acc_d,
+                                    double *mu_ee, double2 *mu_eh, int mom_stride, unsigned int *flags, double tol,
+                                    cudaStream_t s);
+
 // The whole recursion in the registers of thread-block clusters (cluster.cu).
 constexpr int kMaxCluster = 16;  // above 8 it takes CTAs that fill their SMs and a GPC of that many
 constexpr int kClusterSmem = 226 * 1024;  // dynamic shared memory a CTA may ask for
