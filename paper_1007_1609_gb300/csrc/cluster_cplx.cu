@@ -52,7 +52,7 @@ bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int nc
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int TX = (Lx + 3) / 4, TY = (Ly + 1) / 2, pairs = (ncols + kCols - 1) / kCols;
-  const double warp_cycles = nnn ? (bond ? 355.0 : 285.0) : (bond ? 255.0 : 215.0);
+  const double wide = nnn ? (bond ? 355.0 : 285.0) : (bond ? 255.0 : 215.0);
   double best = 0.0;
   for (int cluster = 1; cluster <= kMaxCluster && cluster <= TY; ++cluster) {
     const int rows = (TY + cluster - 1) / cluster, threads = (TX * rows + 31) / 32 * 32 * kCols;
@@ -66,6 +66,7 @@ bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int nc
     const int per_sm = std::max(1, std::min(12 / nw, static_cast<int>(kClusterSmem / (q.smem + 4096))));
     const long long rounds = (pairs + slots - 1) / slots, ctas = static_cast<long long>(pairs) * cluster;
     const int busy = static_cast<int>(std::min<long long>(per_sm, (ctas + sms - 1) / sms));
+    const double warp_cycles = threads > 256 ? wide : 0.78 * wide;  // (the two kernels of cluster_cplx.cuh)
     const double cost = static_cast<double>(rounds) *
                         (900.0 + 250.0 * std::log2(static_cast<double>(cluster)) + warp_cycles * busy * nw);
     if (best == 0.0 || cost < best) {
@@ -78,8 +79,8 @@ bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int nc
   // vector.  Streamed -> on chip, ms, eight hoppings and bond pairing, M = 400: 40 x 36,
   // 400 columns: 6.0 -> 2.3; 64 x 64: 9.3 -> 5.5; 96 x 96: 18.3 -> 9.8; 1000 columns:
   // 41.8 -> 28.3; 120 x 120: 57.2 -> 48.5; 100 x 98: 45.0 -> 42.2.  Clusters of 13 to 16 CTAs
-  // fit the chip only seven times (112 of the 152 SMs), and many columns of them stay
-  // streamed (128 x 128, 800 columns, M = 200: 31.7 ms, 33.4 on chip).
+  // fit the chip only seven times (112 of the 152 SMs): 128 x 128, 512 columns: 31.5 -> 30.8, and
+  // more of them stay streamed.
   return best > 0.0 && best < 21000.0 + 0.0165 * Lx * Ly * ncols;
 }
 

@@ -17,17 +17,21 @@
 //
 // Bound: shared memory.  A tile takes 68 quads a step (52 of coefficients, 16 of the
 // ring) with eight hoppings and bond pairing, 272 wavefronts of its warp: at 64 x 64
-// (four CTAs, eight warps an SM) 2,500 of a step's 4,200 cycles, the packed
+// (four CTAs, eight warps an SM) 2,500 of a step's 3,560 cycles, the packed
 // multiply-adds 1,600; the rest is the chain load - multiply-add - store - barrier,
-// which two warps a scheduler do not hide.  Both start vectors in one thread read the
-// coefficients once for two (50 quads a vector) but leave one warp a scheduler: 75.3 ms
-// for the currents below.  Streamed kernel -> this one: d-wave vortex lattices, 96 x 96, 512 start
-// sites, M = 1024: 59.8 -> 32.4 ms; bond currents of 64 x 64, M = 512: 75.1 -> 63.8 ms;
-// Green's functions of 128 x 128, 16 x 256, M = 1024: 42.1 -> 35.1 ms (28 of them the
+// which two warps a scheduler do not hide.  A store holds back the loads after it, so
+// CTAs of up to 256 threads, which may use 255 registers each, publish a tile when all of
+// it is formed (currents below: 63.8 -> 54.0 ms); wider ones spill that way and
+// publish each column of sites (33.4 ms for the vortex lattice when two are held).
+// Both start vectors in one thread read the coefficients once for two (50 quads a
+// vector) but leave one warp a scheduler: 75.3 ms for the currents.
+// Streamed kernel -> this one: d-wave vortex lattices, 96 x 96, 512 start sites,
+// M = 1024: 59.8 -> 32.4 ms; bond currents of 64 x 64, M = 512: 75.1 -> 54.0 ms;
+// Green's functions of 128 x 128, 16 x 256 sites, M = 1024: 17.0 -> 9.8 ms (3.4 of them the
 // contraction with the energies).  The sums are those of the streamed kernels in
 // their order: the same moments bit for bit.  (Starting from e u - u_old instead of
-// u_old takes six registers fewer a site and 59.7 ms for the currents, but rounds
-// differently: 7.7e-7 from 64 bits instead of 7.1e-7 for the Green's functions.)
+// u_old takes six registers fewer a site and 6 % less time, but rounds differently:
+// 7.7e-7 from 64 bits instead of 7.1e-7 for the Green's functions.)
 #pragma once
 
 #include "cluster.cuh"
@@ -40,6 +44,7 @@ constexpr int kCols = 2;                      // start vectors of a cluster at a
 constexpr int kCxSet = kCx * kCy * kCols;     // quads of one set of published sites
 constexpr int kCxRec = 2 * kCxSet + 1;        // quads of a tile's record (two sets; odd, as in Record)
 constexpr int kCxChunk = 32;                  // coefficients C_m staged at a time
+constexpr int kCxNarrow = 256;                // threads up to which a CTA may use 255 registers each
 constexpr int kCxPlaces = 512;                // targets (of all start vectors) whose place is kept
 
 __device__ __forceinline__ F2 pairs(float x) { return f2pack(x, x); }
@@ -98,8 +103,8 @@ struct Update {
   }
 };
 
-template <bool NNN, bool BOND>
-__global__ void __launch_bounds__(384, 1) cluster_cplx_kernel(CplxClusterArgs a) {
+template <bool NNN, bool BOND, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? 384 : kCxNarrow, 1) cluster_cplx_kernel(CplxClusterArgs a) {
   extern __shared__ __align__(16) unsigned char raw[];
   __shared__ __align__(8) unsigned long long bar_mem;
   __shared__ double ctab[2][kCxChunk];     // C_m of the current and the next chunk of moments
@@ -270,7 +275,6 @@ __global__ void __launch_bounds__(384, 1) cluster_cplx_kernel(CplxClusterArgs a)
           gd1 = gd2;
         }
         w.finish(on.r0, m0, ou[0][c], ov[0][c]);
-        publish(0, c, ou[0][c], ov[0][c], wr);
         tl0 = tf;
         bl0 = bf;
       }
@@ -297,7 +301,6 @@ __global__ void __launch_bounds__(384, 1) cluster_cplx_kernel(CplxClusterArgs a)
           go1 = go2;
         }
         w.finish(on.r0, m1, ou[1][c], ov[1][c]);
-        publish(1, c, ou[1][c], ov[1][c], wr);
         tl1 = tf;
         bl1 = bf;
       }
@@ -307,6 +310,16 @@ __global__ void __launch_bounds__(384, 1) cluster_cplx_kernel(CplxClusterArgs a)
       p0 = p1;
       d1 = d2;
       p1 = p2;
+      if (WIDE) {
+        publish(0, c, ou[0][c], ov[0][c], wr);
+        publish(1, c, ou[1][c], ov[1][c], wr);
+      }
+    }
+    if (!WIDE) {
+#pragma unroll
+      for (int r = 0; r < kCy; ++r)
+#pragma unroll
+        for (int c = 0; c < kCx; ++c) publish(r, c, ou[r][c], ov[r][c], wr);
     }
   };
 
@@ -481,7 +494,7 @@ __global__ void __launch_bounds__(384, 1) cluster_cplx_kernel(CplxClusterArgs a)
 
 template <bool NNN, bool BOND>
 int cplx_slots_one(const ClusterPlan &p) {
-  auto k = cluster_cplx_kernel<NNN, BOND>;
+  auto k = p.threads > kCxNarrow ? cluster_cplx_kernel<NNN, BOND, true> : cluster_cplx_kernel<NNN, BOND, false>;
   Launch<4, 0> l(p);
   int n = 0;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kCplxClusterSmem);
@@ -499,7 +512,8 @@ cudaError_t cplx_launch_one(const CplxClusterArgs &a, const ClusterPlan &p, int 
   Launch<4, 0> l(p);
   l.cfg.gridDim = dim3(clusters * p.cluster);
   l.cfg.stream = s;
-  return cudaLaunchKernelEx(&l.cfg, cluster_cplx_kernel<NNN, BOND>, a);
+  auto k = p.threads > kCxNarrow ? cluster_cplx_kernel<NNN, BOND, true> : cluster_cplx_kernel<NNN, BOND, false>;
+  return cudaLaunchKernelEx(&l.cfg, k, a);
 }
 
 }  // namespace
