@@ -23,7 +23,7 @@ namespace {
 
 constexpr int kRecord = 33, kCols = 2, kMaxThreads = 384;  // as in cluster_cplx.cuh
 
-// p.rag: nnn + 2 bond
+// p.rag: nnn + 2 bond + 4 for periodic sides that the tiles do not divide
 int slots_of(const ClusterPlan &p) {
   static std::mutex mutex;
   static std::map<std::tuple<int, int, int, int, size_t>, int> known;
@@ -33,10 +33,11 @@ int slots_of(const ClusterPlan &p) {
   const auto key = std::make_tuple(dev, p.rag, p.cluster, p.threads, p.smem);
   const auto it = known.find(key);
   if (it != known.end()) return it->second;
-  const int n = p.rag == 0   ? cplx_slots_0_0(p)
-                : p.rag == 1 ? cplx_slots_1_0(p)
-                : p.rag == 2 ? cplx_slots_0_1(p)
-                             : cplx_slots_1_1(p);
+  const int kind = p.rag & 3;
+  const int n = kind == 0   ? cplx_slots_0_0(p)
+                : kind == 1 ? cplx_slots_1_0(p)
+                : kind == 2 ? cplx_slots_0_1(p)
+                            : cplx_slots_1_1(p);
   return known[key] = n;
 }
 
@@ -47,7 +48,8 @@ int slots_of(const ClusterPlan &p) {
 // the warps on an SM; fitted to 32 .. 800 columns of 16 x 16 .. 140 x 120 sites, within 15 %.
 // Falls short (false) where the streamed kernels are expected to be faster.
 bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int ncols, ClusterPlan *p, int *clusters) {
-  if ((px && Lx % 4) || (py && Ly % 2) || ncols < 1) return false;
+  if (ncols < 1) return false;
+  const int rag = (px && Lx % 4) || (py && Ly % 2) ? 4 : 0;
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -57,7 +59,7 @@ bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int nc
   for (int cluster = 1; cluster <= kMaxCluster && cluster <= TY; ++cluster) {
     const int rows = (TY + cluster - 1) / cluster, threads = (TX * rows + 31) / 32 * 32 * kCols;
     if ((TY + rows - 1) / rows != cluster || threads > kMaxThreads) continue;
-    ClusterPlan q{2, cluster, rows, threads, nnn + 2 * bond,
+    ClusterPlan q{2, cluster, rows, threads, nnn + 2 * bond + rag,
                   static_cast<size_t>(TX * rows + (cluster > 1 ? TX : 0) + 1) * 2 * kRecord * 16};
     if (q.smem > kCplxClusterSmem) continue;
     const int slots = slots_of(q);
@@ -66,7 +68,7 @@ bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int nc
     const int per_sm = std::max(1, std::min(12 / nw, static_cast<int>(kClusterSmem / (q.smem + 4096))));
     const long long rounds = (pairs + slots - 1) / slots, ctas = static_cast<long long>(pairs) * cluster;
     const int busy = static_cast<int>(std::min<long long>(per_sm, (ctas + sms - 1) / sms));
-    const double warp_cycles = threads > 256 ? wide : 0.78 * wide;  // (the two kernels of cluster_cplx.cuh)
+    const double warp_cycles = (threads > 256 ? wide : 0.78 * wide) * (rag ? 1.1 : 1.0);  // (the two kernels of cluster_cplx.cuh)
     const double cost = static_cast<double>(rounds) *
                         (900.0 + 250.0 * std::log2(static_cast<double>(cluster)) + warp_cycles * busy * nw);
     if (best == 0.0 || cost < best) {
@@ -81,7 +83,9 @@ bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int nc
   // 41.8 -> 28.3; 120 x 120: 57.2 -> 48.5; 100 x 98: 45.0 -> 42.2.  Clusters of 13 to 16 CTAs
   // fit the chip only seven times (112 of the 152 SMs): 128 x 128, 512 columns: 31.5 -> 30.8, and
   // more of them stay streamed.
-  return best > 0.0 && best < 21000.0 + 0.0165 * Lx * Ly * ncols;
+  // Ragged periodic sides: 33 x 33, 512 columns: 6.0 -> 1.6; 75 x 90, 1000: 35.2 -> 19.0; 98 x 98: 41.4 ->
+  // 36.7; 121 x 119 would take 1.08 of the streamed time, so they are given a margin.
+  return best > 0.0 && best * (rag ? 1.15 : 1.0) < 21000.0 + 0.0165 * Lx * Ly * ncols;
 }
 
 cudaError_t launch_cluster_cplx(CplxClusterArgs a, int bond, const ClusterPlan &p, int clusters, cudaStream_t s) {

@@ -103,7 +103,7 @@ struct Update {
   }
 };
 
-template <bool NNN, bool BOND, bool WIDE>
+template <bool NNN, bool BOND, bool WIDE, bool RAG>
 __global__ void __launch_bounds__(WIDE ? 384 : kCxNarrow, 1) cluster_cplx_kernel(CplxClusterArgs a) {
   extern __shared__ __align__(16) unsigned char raw[];
   __shared__ __align__(8) unsigned long long bar_mem;
@@ -160,6 +160,15 @@ __global__ void __launch_bounds__(WIDE ? 384 : kCxNarrow, 1) cluster_cplx_kernel
     return (CS > 1 ? record(ghost + x) : record((gy < 0 ? TY - 1 : 0) * TX + x)) + k * 16;
   };
   const unsigned own = (act ? record(tt) : record(nil)) + k * 16;
+  // Periodic sides that the tiles do not divide (RAG): the last tiles have rx columns or one row.  What
+  // lies beyond it takes the place of the missing one: rt's column 0 of column rx, up's row 0 of row 1.
+  // Seen from the first tiles, the last ones' column rx - 1 (row 0) is the neighbour: the addresses of lf,
+  // ul and dl (dn, dl and dr) move by back_x (back_y) sites.
+  const int rx = Lx - kCx * (TX - 1);
+  const int rsel = RAG && a.px && tx == TX - 1 ? rx : kCx;
+  const bool end_y = RAG && a.py && (Ly & 1) && act && ty == TY - 1;
+  const int back_x = RAG && a.px && tx == 0 ? rx - kCx : 0;
+  const int back_y = RAG && a.py && (Ly & 1) && CS == 1 && ty == 0 ? -kCx : 0;
   const unsigned lf = act ? tile(-1, 0) : own, rt = act ? tile(1, 0) : own, up = act ? tile(0, 1) : own;
   const unsigned dn = act ? tile(0, -1) : own, ul = act ? tile(-1, 1) : own, ur = act ? tile(1, 1) : own;
   const unsigned dl = act ? tile(-1, -1) : own, dr = act ? tile(1, -1) : own;
@@ -170,9 +179,9 @@ __global__ void __launch_bounds__(WIDE ? 384 : kCxNarrow, 1) cluster_cplx_kernel
     if (tyl == 0 && (ty > 0 || a.py)) push_dn = remote(record(ghost + tx) + k * 16, rank > 0 ? rank - 1 : CS - 1);
   }
   // coefficients of the tile's sites: quads (t_+x, t_+y), (t_+x+y, t_-x+y), (B_+x, B_+y), (e, Delta)
-  auto load_coef = [&](unsigned rec, int gx, int gy, int r) {
+  auto load_coef = [&](unsigned rec, int gx, int gy, int r, int skip = 0) {
     for (int c = 0; c < kCx; ++c) {
-      const int x = gx + c, y = gy + r;
+      const int x = gx + c, y = gy + r - skip;
       if (x >= Lx || y >= Ly) continue;
       auto field = [&](int k) {
         return *reinterpret_cast<const float2 *>(a.params + ((static_cast<size_t>(y) * kCplxFields + k) * Lx + x) * 2);
@@ -188,7 +197,8 @@ __global__ void __launch_bounds__(WIDE ? 384 : kCxNarrow, 1) cluster_cplx_kernel
   if (act) load_coef(record(tt), x0, y0, k);
   if (CS > 1 && t < TX) {  // of the row below this CTA's
     const int gy = rank * R - 1;
-    if (gy >= 0 || a.py) load_coef(record(ghost + t), kCx * t, kCy * (gy < 0 ? TY - 1 : gy), 1);
+    // (the last row of tiles may have one row of sites: it takes the place of the second)
+    if (gy >= 0 || a.py) load_coef(record(ghost + t), kCx * t, kCy * (gy < 0 ? TY - 1 : gy), 1, RAG && gy < 0 ? Ly & 1 : 0);
   }
   if (CS > 1) {
     cluster_arrive();
@@ -202,7 +212,11 @@ __global__ void __launch_bounds__(WIDE ? 384 : kCxNarrow, 1) cluster_cplx_kernel
   auto publish = [&](int r, int c, F2 u, F2 v, int wr) {
     const int at_ = wr + (r * kCx + c) * kCols * 16;
     sts4(own + at_, u, v);
-    if (r == 1 && push_up) push4(push_up + at_, u, v);
+    if (RAG && end_y) {
+      if (r == 0 && push_up) push4(push_up + at_ + kCx * kCols * 16, u, v);
+    } else if (r == 1 && push_up) {
+      push4(push_up + at_, u, v);
+    }
     if (r == 0 && push_dn) push4(push_dn + at_, u, v);
   };
   // (o) = 2 H~ (z) - (o), published as it is formed; both rows of a column of sites at once
@@ -211,66 +225,77 @@ __global__ void __launch_bounds__(WIDE ? 384 : kCxNarrow, 1) cluster_cplx_kernel
     if (!act) return;
     auto far = [&](unsigned rec, int r, int c) { return lds4(rec + rd + (r * kCx + c) * kCols * 16); };
     auto coef = [&](unsigned rec, int r, int c, int q) { return ldc(rec + coff + (r * kCx + c) * 64 + q * 16); };
+    // (the same in tiles seen across a ragged edge)
+    const unsigned lv = lf + back_x * kCols * 16, lc = lf + back_x * 64, ulv = ul + back_x * kCols * 16;
+    const unsigned dnv = dn + back_y * kCols * 16, dnc = dn + back_y * 64, drv = dr + back_y * kCols * 16, drc = dr + back_y * 64;
+    const unsigned dlv = dl + (back_x + back_y) * kCols * 16, dlc = dl + (back_x + back_y) * 64;
     // columns x - 1 and x of the rows below (d) and above (p) the tile, and of the tile's own rows 0 and 1
-    Quad d0{}, p0{}, l0 = far(lf, 0, kCx - 1), l1 = far(lf, 1, kCx - 1);
+    Quad d0{}, p0{}, l0 = far(lv, 0, kCx - 1), l1 = far(lv, 1, kCx - 1);
     if (NNN) {
-      d0 = far(dl, 1, kCx - 1);
-      p0 = far(ul, 0, kCx - 1);
+      d0 = far(dlv, 1, kCx - 1);
+      p0 = far(ulv, 0, kCx - 1);
     }
-    Quad d1 = far(dn, 1, 0), p1 = far(up, 0, 0);
+    Quad d1 = far(dnv, 1, 0), p1 = far(up, 0, 0);
     // column x - 1's forward x hopping and bond of rows 0 and 1; the diagonal hoppings of the
     // row below and of row 0 at x - 1 and x
-    Coef tl0 = coef(lf, 0, kCx - 1, 0), tl1 = coef(lf, 1, kCx - 1, 0), bl0{}, bl1{}, gd0{}, gd1{}, go0{}, go1{};
+    Coef tl0 = coef(lc, 0, kCx - 1, 0), tl1 = coef(lc, 1, kCx - 1, 0), bl0{}, bl1{}, gd0{}, gd1{}, go0{}, go1{};
     if (BOND) {
-      bl0 = coef(lf, 0, kCx - 1, 2);
-      bl1 = coef(lf, 1, kCx - 1, 2);
+      bl0 = coef(lc, 0, kCx - 1, 2);
+      bl1 = coef(lc, 1, kCx - 1, 2);
     }
     if (NNN) {
-      gd0 = coef(dl, 1, kCx - 1, 1);
-      gd1 = coef(dn, 1, 0, 1);
-      go0 = coef(lf, 0, kCx - 1, 1);
+      gd0 = coef(dlc, 1, kCx - 1, 1);
+      gd1 = coef(dnc, 1, 0, 1);
+      go0 = coef(lc, 0, kCx - 1, 1);
       go1 = coef(own, 0, 0, 1);
     }
 #pragma unroll
     for (int c = 0; c < kCx; ++c) {
       const int cn = c < kCx - 1 ? c + 1 : c;
       const bool last = c == kCx - 1;
+      const bool wrap = RAG && !last && c + 1 == rsel;  // column x + 1 is rt's first
       const Quad m0{zu[0][c], zv[0][c]}, m1{zu[1][c], zv[1][c]};
       Quad r0{zu[0][cn], zv[0][cn]}, r1{zu[1][cn], zv[1][cn]}, d2{}, p2{};  // column x + 1
       if (last) {
         r0 = far(rt, 0, 0);
         r1 = far(rt, 1, 0);
         if (NNN) {
-          d2 = far(dr, 1, 0);
+          d2 = far(drv, 1, 0);
           p2 = far(ur, 0, 0);
         }
       } else {
-        d2 = far(dn, 1, cn);
-        p2 = far(up, 0, cn);
+        d2 = far(wrap ? drv - cn * kCols * 16 : dnv, 1, cn);
+        p2 = far(wrap ? ur - cn * kCols * 16 : up, 0, cn);
+        if (wrap) {
+          r0 = far(rt, 0, 0);
+          r1 = far(rt, 1, 0);
+        }
       }
+      // row 0's neighbours above: row 1, or what lies beyond a last row
+      const Quad a0 = RAG && end_y ? p0 : l1, a1 = RAG && end_y ? p1 : m1, a2 = RAG && end_y ? p2 : r1;
       {  // row 0
-        const Coef on = coef(own, 0, c, 3), tf = coef(own, 0, c, 0), td = coef(dn, 1, c, 0);
+        const Coef on = coef(own, 0, c, 3), tf = coef(own, 0, c, 0), td = coef(dnc, 1, c, 0);
         Update w(BOND, on, m0, ou[0][c]);
         Coef bf{}, bd{};
         if (BOND) {
           bf = coef(own, 0, c, 2);
-          bd = coef(dn, 1, c, 2);
+          bd = coef(dnc, 1, c, 2);
         }
         w.hop(tf.r0, tf.i0, r0);
         if (BOND) w.pair(bf.r0, bf.i0, r0);
         w.hop(tl0.r0, -tl0.i0, l0);
         if (BOND) w.pair(bl0.r0, bl0.i0, l0);
-        w.hop(tf.r1, tf.i1, m1);
-        if (BOND) w.pair(bf.r1, bf.i1, m1);
+        w.hop(tf.r1, tf.i1, a1);
+        if (BOND) w.pair(bf.r1, bf.i1, a1);
         w.hop(td.r1, -td.i1, d1);
         if (BOND) w.pair(bd.r1, bd.i1, d1);
         if (NNN) {
           // (t_+x+y, t_-x+y) of the site; backward, the lower left site's t_+x+y and the lower right's t_-x+y
-          const Coef gd2 = last ? coef(dr, 1, 0, 1) : coef(dn, 1, cn, 1);
-          w.hop(go1.r0, go1.i0, r1);
+          const Coef gd2 = last ? coef(drc, 1, 0, 1) : coef(wrap ? drc - cn * 64 : dnc, 1, cn, 1);
+          w.hop(go1.r0, go1.i0, a2);
           w.hop(gd0.r0, -gd0.i0, d0);
           w.hop(gd2.r1, -gd2.i1, d2);
-          w.hop(go1.r1, go1.i1, l1);
+          w.hop(go1.r1, go1.i1, a0);
           gd0 = gd1;
           gd1 = gd2;
         }
@@ -292,7 +317,7 @@ __global__ void __launch_bounds__(WIDE ? 384 : kCxNarrow, 1) cluster_cplx_kernel
         w.hop(tl0.r1, -tl0.i1, m0);
         if (BOND) w.pair(bl0.r1, bl0.i1, m0);
         if (NNN) {
-          const Coef gp = coef(own, 1, c, 1), go2 = last ? coef(rt, 0, 0, 1) : coef(own, 0, cn, 1);
+          const Coef gp = coef(own, 1, c, 1), go2 = last ? coef(rt, 0, 0, 1) : coef(wrap ? rt - cn * 64 : own, 0, cn, 1);
           w.hop(gp.r0, gp.i0, p2);
           w.hop(go0.r0, -go0.i0, l0);
           w.hop(go2.r1, -go2.i1, r0);
@@ -493,8 +518,14 @@ __global__ void __launch_bounds__(WIDE ? 384 : kCxNarrow, 1) cluster_cplx_kernel
 }
 
 template <bool NNN, bool BOND>
+auto cplx_kernel_of(const ClusterPlan &p) {  // p.rag bit 2: ragged periodic sides
+  if (p.rag & 4) return p.threads > kCxNarrow ? cluster_cplx_kernel<NNN, BOND, true, true> : cluster_cplx_kernel<NNN, BOND, false, true>;
+  return p.threads > kCxNarrow ? cluster_cplx_kernel<NNN, BOND, true, false> : cluster_cplx_kernel<NNN, BOND, false, false>;
+}
+
+template <bool NNN, bool BOND>
 int cplx_slots_one(const ClusterPlan &p) {
-  auto k = p.threads > kCxNarrow ? cluster_cplx_kernel<NNN, BOND, true> : cluster_cplx_kernel<NNN, BOND, false>;
+  auto k = cplx_kernel_of<NNN, BOND>(p);
   Launch<4, 0> l(p);
   int n = 0;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kCplxClusterSmem);
@@ -512,7 +543,7 @@ cudaError_t cplx_launch_one(const CplxClusterArgs &a, const ClusterPlan &p, int 
   Launch<4, 0> l(p);
   l.cfg.gridDim = dim3(clusters * p.cluster);
   l.cfg.stream = s;
-  auto k = p.threads > kCxNarrow ? cluster_cplx_kernel<NNN, BOND, true> : cluster_cplx_kernel<NNN, BOND, false>;
+  auto k = cplx_kernel_of<NNN, BOND>(p);
   return cudaLaunchKernelEx(&l.cfg, k, a);
 }
 
