@@ -38,6 +38,18 @@ UNIT = "vector-steps/s"
 L, M, SEED = 128, 1024, 1001
 # per vector element and step: the stencil's 6 FMAs and half of a site's 6 product FMAs (FMA = 2 flops)
 FP64_FLOPS_PER_ELEMENT_STEP = 18.0
+FP32_FLOPS_PER_ELEMENT_STEP = 18.0
+# An FP32 adjoint advances an element twice (forward, reversed) at 12 flops, adds the source at 2 and
+# the gradient sums at 10.
+ADJOINT_FLOPS_PER_ELEMENT_STEP = 36.0
+L2_FLUSH_BYTES = 256 << 20
+
+
+def on_chip_roofline(flops, ms, peak, note):
+    """Roofline of a recursion that keeps its vectors in registers: FP32 multiply-adds."""
+    tf = flops / (ms * 1e-3) / 1e12
+    return {"bound": "alu", "achieved": tf, "peak": peak, "unit": "TFLOP/s", "frac": tf / peak if peak else None,
+            "peak_kind": "measured (cbdg_measure_peak, FP32 FMA)", "note": note}
 
 
 def kernel_source_digest(sources):
@@ -254,8 +266,15 @@ def run_gb300(args):
     lat = cbdg.Lattice(p, precision="fp32", stream=stream)
     if args.temporal is not None:
         lat.set_option(cbdg.CBDG_OPT_TEMPORAL_STEPS, args.temporal)
+    flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device=dev)
+
+    def flushed_step():
+        """One iteration after a write of a buffer larger than L2 (inside the timed region)."""
+        with torch.cuda.stream(stream):
+            flush.zero_()
+        return lat.scf_step(p.T, p.M, p.mix)
     for _ in range(args.warmup):
-        lat.scf_step(p.T, p.M, p.mix)
+        flushed_step()
     # the production path: every iteration after the second is a CUDA-graph replay
     cbdg.cbdg_launch_count(lat.handle, reset=True)
     e0 = torch.cuda.Event(enable_timing=True)
@@ -263,7 +282,7 @@ def run_gb300(args):
     barrier()
     with ClockSampler(local) as clk:
         e0.record(stream)
-        diffs = [lat.scf_step(p.T, p.M, p.mix) for _ in range(args.steps)]
+        diffs = [flushed_step() for _ in range(args.steps)]
         e1.record(stream)
         torch.cuda.synchronize()
     barrier()
@@ -304,6 +323,8 @@ def run_gb300(args):
         barrier()
         t0 = time.perf_counter()
         for _ in range(args.steps):
+            with torch.cuda.stream(stream):
+                flush.zero_()
             cbdg.cbdg_set_delta(lat_e.handle, host_delta)
             cbdg.cbdg_scf_step(lat_e.handle, p.T, p.M, p.mix)
             cbdg.cbdg_get_delta(lat_e.handle, host_out)
@@ -347,6 +368,14 @@ def run_gb300(args):
                     "share_of_step": step_ms / prof_ms if prof_ms else None}
         extra = {}
         ap = arith_peaks(cbdg, torch, stream, local)
+        if step_n and not step_bytes:  # the vectors never left the registers
+            elements = 2 * p.N * p.N * ((p.M + 1) // 2 - 1) * prof_iters
+            roofline.update(on_chip_roofline(
+                FP32_FLOPS_PER_ELEMENT_STEP * elements, step_ms, ap["fp32_fma"]["tflops"],
+                "whole recursion of an iteration in one launch of persistent thread-block clusters"))
+            roofline.update({"kernel": "cluster_kernel: FP32 recursion in the registers of thread-block clusters",
+                             "traffic": None, "traffic_source": None, "algorithmic_bytes_per_launch": 0,
+                             "steps_per_pass": (p.M + 1) // 2 - 1})
         extra["arith_peaks"] = ap
         if not args.no_fp64:
             extra["fp64"] = fp64_leg(p, stream, cbdg, torch, units_per_step, fp64_peak=ap["fp64_fma"]["tflops"])
@@ -378,8 +407,8 @@ def run_gb300(args):
                                    "start vectors, FP32 recursion with FP64 folds",
                        "step": "one self-consistency iteration",
                        "units_per_step": units_per_step,
-                       "l2": "no flush: the two recursion vectors are 2 x 2.1 GB per rank, "
-                             "far larger than the 126 MB L2",
+                       "l2": f"flushed before every iteration: a {L2_FLUSH_BYTES >> 20} MB buffer is written, "
+                             "inside the timed region",
                        "parallelism": f"replicas x{world}"},
             "roofline": roofline,
             "cpu_baseline": cpu,
@@ -454,6 +483,14 @@ def leg_contraction(cbdg, torch, stream, shape=(65536, 2048, 512), tf32_peak=Non
                                  "the method's 2 m n k"}}
 
 
+def recursion_roofline(sms, sb, hbm, note):
+    """Roofline of profiled recursion launches by the bytes of their vectors; None where they move none."""
+    if not sb or not sms:
+        return None
+    gbs = sb / (sms * 1e-3) / 1e9
+    return {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm, "note": note}
+
+
 def leg_dwave(cbdg, wl, stream, hbm, columns=4096):
     """General recursion step (complex64, t', bond pairing, Peierls field) on
     the 256x256 vortex lattice, a chunk of `columns` start sites."""
@@ -469,9 +506,8 @@ def leg_dwave(cbdg, wl, stream, hbm, columns=4096):
     tile = lat.last_tile()
     lat.close()
     return {"lattice": "256x256 periodic, t'=-0.3, 2 h/2e flux, bond pairing, complex64",
-            "columns": int(columns), "launches": sn, "avg_launch_ms": sms / sn, "tile": list(tile),
-            "roofline": {"bound": "hbm", "achieved": sb / (sms * 1e-3) / 1e9, "peak": hbm,
-                         "unit": "GB/s", "frac": sb / (sms * 1e-3) / 1e9 / hbm}}
+            "columns": int(columns), "launches": sn, "avg_launch_ms": sms / max(sn, 1), "tile": list(tile),
+            "roofline": recursion_roofline(sms, sb, hbm, "step_cplx_kernel (direct mode)")}
 
 
 def leg_ensemble(cbdg, wl, stream, samples=256):
@@ -491,9 +527,11 @@ def leg_ensemble(cbdg, wl, stream, samples=256):
     steps = (512 + 1) // 2 - 1
     streams = 4 * (steps // 3) + 3 * (steps % 3)
     algo_bytes = sum(streams * 2 * p.N * 4 * p.N for p in probs)
+    flops = sum(FP32_FLOPS_PER_ELEMENT_STEP * 2 * p.N * p.N * steps for p in probs)
     return {"samples": len(probs), "s_per_iteration": t2 - t1, "first_call_s": t1 - t0,
-            "vector_steps_per_s": units / (t2 - t1), "algorithmic_gbs": algo_bytes / (t2 - t1) / 1e9,
-            "algorithmic_bytes": algo_bytes, "streams_per_column": streams,
+            "vector_steps_per_s": units / (t2 - t1), "tflops": flops / (t2 - t1) / 1e12,
+            # what streamed members (hoppings that differ) would move; those with one hopping run in registers
+            "streamed_bytes": algo_bytes, "streams_per_column": streams,
             "streams_per_column_one_step_per_pass": 3 * steps}
 
 
@@ -535,9 +573,9 @@ def adjoint_streams(M, multi=False):
     return fwd + rec + rev
 
 
-def leg_adjoint(cbdg, wl, stream, hbm):
-    """Gradient of one self-consistency map, 64x64, M = 512 (FP64 and FP32),
-    with the algorithmic bytes of the implemented schedule (adjoint_streams);
+def leg_adjoint(cbdg, wl, stream, hbm, fp32_peak=None):
+    """Gradient of one self-consistency map, 64x64, M = 512 (FP64, and FP32
+    against the FP32 rate);
     and of the general-lattice map (64x64 periodic d-wave lattice with field,
     t' and two vortices: complex64 vectors, one step per launch), FP32."""
     import numpy as np
@@ -559,7 +597,7 @@ def leg_adjoint(cbdg, wl, stream, hbm):
                                     "note": "64x64 d-wave vortex lattice (bond pairing, t', field), complex64; "
                                             "whole backward call over its algorithmic bytes"}
     pg = wl.gradient_case()
-    for prec, es in (("fp64", 8), ("fp32", 4)):
+    for prec in ("fp64", "fp32"):
         lg = cbdg.Lattice(pg, precision=prec, stream=stream)
         d, _ = lg.order_parameter(pg.T, pg.M)
         w = (2.0 * (d.real - pg.extra["target"])).astype(np.complex128)
@@ -570,15 +608,11 @@ def leg_adjoint(cbdg, wl, stream, hbm):
         out[f"{prec}_s"] = dt
         lg.close()
         if prec == "fp32":
-            vb = 2 * pg.N * pg.N * es
-            streams = adjoint_streams(pg.M, multi=True)
-            gbs = streams * vb / dt / 1e9
-            out["fp32_roofline"] = {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s",
-                                    "frac": gbs / hbm, "streams": streams, "vector_bytes": vb,
-                                    "streams_one_step_per_pass": adjoint_streams(pg.M),
-                                    "note": "whole backward call (forward with checkpoints, recomputation and "
-                                            "reverse recursion three steps per pass, accumulation) over its "
-                                            "algorithmic bytes"}
+            flops = ADJOINT_FLOPS_PER_ELEMENT_STEP * 2 * pg.N * pg.N * pg.M
+            out["fp32_roofline"] = on_chip_roofline(
+                flops, dt * 1e3, fp32_peak,
+                "whole backward call: forward and reversed recursion, reverse recursion and gradient sums in the "
+                "registers of thread-block clusters")
     return out
 
 
@@ -631,9 +665,8 @@ def leg_currents(cbdg, wl, torch, stream, hbm):
             "M": p.M, "call_ms": ms, "vector_steps_per_s": units / (ms * 1e-3),
             "step_launches": sn, "avg_step_ms": sms / max(sn, 1), "step_share_of_call": sms / ms,
             "tile": list(tile), "max_abs_J": float(abs(J).max()),
-            "roofline": {"bound": "hbm", "achieved": sb / (sms * 1e-3) / 1e9, "peak": hbm, "unit": "GB/s",
-                         "frac": sb / (sms * 1e-3) / 1e9 / hbm,
-                         "note": "step_cplx_kernel (direct mode), 3 vector streams of 2N x N x 8 B per step"}}
+            "roofline": recursion_roofline(
+                sms, sb, hbm, "step_cplx_kernel (direct mode), 3 vector streams of 2N x N x 8 B per step")}
 
 
 def leg_junction(cbdg, wl, torch, stream, hbm):
@@ -675,9 +708,11 @@ def leg_junction(cbdg, wl, torch, stream, hbm):
             "max_abs_ddelta": diff, "delta_bulk": float(abs(d[L * 150])), "delta_interface": float(abs(d[L * 299])),
             "surface_ldos_s": t3 - t2, "lorentz_lambda": lam, "surface_ldos_at_0": float(rho[:, 100].mean()),
             "steps_per_pass": k, "tile": list(tile), "recursion_launches": sn, "recursion_ms": sms,
-            "roofline": {"bound": "hbm", "achieved": sb / (sms * 1e-3) / 1e9, "peak": hbm, "unit": "GB/s",
-                         "frac": sb / (sms * 1e-3) / 1e9 / hbm,
-                         "note": "recursion kernels over their algorithmic bytes (one start site per layer)"}}
+            "roofline": recursion_roofline(
+                sms, sb, hbm, "recursion kernels over their algorithmic bytes (one start site per layer)")
+            or on_chip_roofline(FP32_FLOPS_PER_ELEMENT_STEP * 2 * p.N * p.Ly * ((p.M + 1) // 2 - 1), sms,
+                                arith_peaks(cbdg, torch, stream)["fp32_fma"]["tflops"],
+                                "cluster_kernel (vectors in registers), one start site per layer")}
 
 
 def leg_green(cbdg, wl, torch, stream, fp64_peak=None):
@@ -685,7 +720,7 @@ def leg_green(cbdg, wl, torch, stream, fp64_peak=None):
     d-wave lattice, M = 1024: 16 start sites (a 4x4 block at the core) x 256
     targets (a 16x16 block) x 512 energies in [-0.5a, 0.5a], device outputs.
     The recursion (16 columns, 1022 steps) is timed by cbdg_green_moments;
-    the FP64 contraction is the difference to cbdg_green_function (weights
+    the exact contraction is the difference to cbdg_green_function (weights
     and two [M] x [M x 512] complex contractions per (site, target))."""
     import numpy as np
     p = wl.currents_dwave(128, 1024)
@@ -724,15 +759,16 @@ def leg_green(cbdg, wl, torch, stream, fp64_peak=None):
     lat.close()
     flops = 2 * 8.0 * ns * nt * M * n_E
     t_con = max(t_all - t_mom, 1e-9)
-    tf = flops / t_con / 1e12
+    # eight base-256 digits an operand, 36 digit products of each real multiply-add
+    tf = 36 * flops / t_con / 1e12
     return {"lattice": "128x128 d-wave vortex lattice, complex64 recursion", "M": M, "sites": ns, "targets": nt,
             "energies": n_E, "moments_s": t_mom, "green_function_s": t_all, "contraction_s": t_con,
-            "roofline": {"bound": "alu", "achieved": tf, "peak": fp64_peak or 1.25, "unit": "TFLOP/s",
-                         "frac": tf / (fp64_peak or 1.25),
-                         "peak_kind": ("measured (cbdg_measure_peak, FP64 FMA)" if fp64_peak
-                                       else "nominal FP64 rate of the profiling recipe's table"),
-                         "note": "green_contract_kernel, FP64 complex multiply-adds (8 flops each), from the call "
-                                 "time difference"}}
+            "fp64_equivalent_tflops": flops / t_con / 1e12,
+            "roofline": {"bound": "tensor", "achieved": tf, "peak": bf16_peak(), "unit": "TFLOP/s",
+                         "frac": tf / bf16_peak() if bf16_peak() else None,
+                         "peak_kind": "measured (cuBLAS bf16 GEMM)",
+                         "note": "digits_contract_kernel: exact FP64 contraction by bf16 digit products, from the "
+                                 "call time difference"}}
 
 
 def scf_to(lat, p, tol, max_iter, torch, err_tol=None):
@@ -815,7 +851,7 @@ def extra_legs(cbdg, wl, torch, stream, hbm, only=None, columns=4096, samples=25
         "contraction": lambda: leg_contraction(cbdg, torch, stream, tf32_peak=ap["tf32_mma"]["tflops"]),
         "dwave": lambda: leg_dwave(cbdg, wl, stream, hbm, columns),
         "ensemble": lambda: leg_ensemble(cbdg, wl, stream, samples),
-        "adjoint": lambda: leg_adjoint(cbdg, wl, stream, hbm),
+        "adjoint": lambda: leg_adjoint(cbdg, wl, stream, hbm, fp32_peak=ap["fp32_fma"]["tflops"]),
         "currents": lambda: leg_currents(cbdg, wl, torch, stream, hbm),
         "junction": lambda: leg_junction(cbdg, wl, torch, stream, hbm),
         "green": lambda: leg_green(cbdg, wl, torch, stream, fp64_peak=ap["fp64_fma"]["tflops"]),
@@ -888,6 +924,9 @@ def fp64_leg(p, stream, cbdg, torch, units_per_step, fp64_peak=None):
     lat.close()
     elements = 2 * p.N * p.N  # rows x columns advanced per launch
     flops = FP64_FLOPS_PER_ELEMENT_STEP * elements * step_n
+    if not step_n:  # in shared memory, one launch: the whole iteration's time
+        flops = FP64_FLOPS_PER_ELEMENT_STEP * elements * ((p.M + 1) // 2 - 1)
+        step_ms = ms
     return {"value": units_per_step / (ms / 1e3), "unit": UNIT, "ms_per_step": ms,
             "dtype": "f64",
             "roofline": {"bound": "alu", "achieved": flops / (step_ms / 1e3) / 1e12,

@@ -232,9 +232,12 @@ cbdg_status cbdg_scf_step(cbdg_lattice *lat, double T, int32_t M, double mix,
  *                               Delta_{j,d^1} = Delta_{i,d} moving together)
  * Any output may be NULL; outputs are host or device arrays.  Real lattices
  * run the real recursion (imaginary parts 0), general ones complex vectors.
- * The forward recursion runs without doubling, keeps checkpoints of
- * (j_{kS}, j_{kS+1}) every S = ceil(sqrt(M)) steps and recomputes each
- * segment during the reverse sweep
+ * FP32 lattices with one real hopping run it in the registers of thread-block
+ * clusters where they fit (M <= 4096, periodic sides multiples of four): pairs
+ * (j_n, j_{n+1}) are kept every 8 steps and the recursion is run backwards
+ * between them.  Elsewhere the forward recursion runs without doubling, keeps
+ * checkpoints of (j_{kS}, j_{kS+1}) every S = ceil(sqrt(M)) steps and recomputes
+ * each segment during the reverse sweep
  *   lam_m = y_m + 2 H~ lam_{m+1} - lam_{m+2},
  * with the source y_m = (U_i/2) C_m conj(g_i) h_i (on-site) or
  * (C_m/8) conj(V_{i,d} g_{i,d} + V_{j,d^1} g_{j,d^1}) h_j on each bond.
@@ -368,7 +371,8 @@ enum {
   CBDG_OPT_TEMPORAL_STEPS = 12,  /* recursion steps K per pass over the vectors (temporal
                                     blocking), 1..4, for real on-site FP32 lattices with open
                                     y edges: one pass reads j_(n-1), j_n and writes
-                                    j_(n+K-1), j_(n+K); 1 = one step per pass; 0 (default) =
+                                    j_(n+K-1), j_(n+K); 1 = one step per pass; 0 (default):
+                                    on chip where CBDG_OPT_RESIDENT allows it, else
                                     3 where each thread holds one lattice site (Lx <= 256 /
                                     (W / 4)) and at slab width 16 up to Lx = 128 (the lean
                                     pass), else 2.  Shapes the multi-step kernel does not
@@ -393,15 +397,19 @@ enum {
                                     autotuning, with a fixed rescale or the stall hook); any
                                     option change or buffer reallocation drops the graph;
                                     0: always launch directly */
-  CBDG_OPT_RESIDENT = 14         /* 1 (default): real on-site lattices whose two vectors per
-                                    column slab, stencil parameters and coefficient table
-                                    fit in one SM's shared memory (about 2300 sites in FP64,
-                                    4700 in FP32) run the whole recursion on chip, one
-                                    launch per pass (unless a tile option, autotuning or the
-                                    stall hook is set); 0: the streamed kernels */
+  CBDG_OPT_RESIDENT = 14         /* 1 (default): recursions whose vectors fit on chip run
+                                    there, one launch per pass over the start sites (unless
+                                    a tile option, autotuning or the stall hook is set):
+                                    FP32 real on-site lattices with one hopping in the
+                                    registers of thread-block clusters (up to about 160,000
+                                    sites); general FP32 lattices (up to about 20,000 sites)
+                                    likewise, where that is expected to be faster; other real
+                                    on-site lattices in one SM's shared memory (about 2300
+                                    sites in FP64, 4000 with one hopping, 4700 in FP32);
+                                    0: the streamed kernels */
 };
 /* Read-only (cbdg_get_option): the tile of the last recursion pass, packed as
- * slab width | depth << 16 | row split << 32. */
+ * slab width | depth << 16 | row split << 32; depth 0: the pass ran on chip. */
 enum { CBDG_INFO_LAST_TILE = 100 };
 /* Read-only: recursion steps per pass (K) used by the last pass. */
 enum { CBDG_INFO_LAST_TEMPORAL = 101 };
@@ -410,16 +418,17 @@ cbdg_status cbdg_get_option(cbdg_lattice *lat, int32_t option, int64_t *value);
 
 /* Accumulated device time of the recursion-step kernel since the last reset
  * (CBDG_OPT_PROFILE must be on): total milliseconds, number of launches and
- * algorithmic bytes (read j_n, read j_{n-1}, write j_{n+1}) summed over the
- * launches.  reset != 0 clears the counters after reading. */
+ * algorithmic bytes (read j_n, read j_{n-1}, write j_{n+1}; 0 for a recursion in
+ * registers, whose one launch counts all its steps) summed over the launches.  reset != 0 clears the counters after reading. */
 cbdg_status cbdg_profile_read(cbdg_lattice *lat, double *step_ms, int64_t *step_launches,
                               double *step_bytes, int32_t reset);
 
 /* Ensembles: many independent lattices (disorder realisations of uneven
  * size) iterated to self-consistency together.  Every member: real on-site
  * pairing, 4 directions, open edges, CBDG_FP32_MIXED, sides <= 128, and one
- * shared mu and U.  Each iteration is one persistent launch over (sample,
- * 16-column slab) work items plus small batched kernels (rescale, Fermi
+ * shared mu and U.  An iteration runs the members with one real hopping in the registers
+ * of thread-block clusters, a launch each in parallel branches, the others in one persistent
+ * launch over (sample, 16-column slab) work items, plus small batched kernels (rescale, Fermi
  * coefficients by K-node quadrature, parameters, mixing, convergence),
  * captured once as a CUDA graph and replayed.  Not in the paper: a batching
  * layer over its self-consistency loop (paragraph after Eq. 20). */
