@@ -461,7 +461,7 @@ cbdg_status run_cplx_on_chip(cbdg_lattice *L, const void *params, const int32_t 
   const int bond = L->pairing == CBDG_BOND_V ? 1 : 0;
   *ran = false;
   if (!on_chip_options(L) || n_sites < 1 ||
-      !plan_cluster_cplx(L->Lx, L->Ly, L->px, L->py, L->n_dirs == 8, bond, n_sites, &plan, &clusters))
+      !plan_cluster_cplx(L->Lx, L->Ly, L->px, L->py, L->n_dirs == 8, bond, n_sites, c.n_t, &plan, &clusters))
     return CBDG_OK;
   c.params = static_cast<const float *>(params);
   c.scal = L->scal.as<double>();

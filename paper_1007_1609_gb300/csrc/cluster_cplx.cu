@@ -45,9 +45,9 @@ int slots_of(const ClusterPlan &p) {
 
 // Cycles of a step of all columns, by clusters: a round takes 900 for the chain through shared
 // memory, 250 for each doubling of the cluster (its barrier) and the shared-memory wavefronts of
-// the warps on an SM; fitted to 32 .. 800 columns of 16 x 16 .. 140 x 120 sites, within 15 %.
+// the warps on an SM, 1500 every pass of the threads over the targets after the first; fitted to 32 .. 800 columns of 16 x 16 .. 140 x 120 sites, within 15 %.
 // Falls short (false) where the streamed kernels are expected to be faster.
-bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int ncols, ClusterPlan *p, int *clusters) {
+bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int ncols, int n_t, ClusterPlan *p, int *clusters) {
   if (ncols < 1) return false;
   const int rag = (px && Lx % 4) || (py && Ly % 2) ? 4 : 0;
   int dev = 0, sms = 152;
@@ -70,7 +70,8 @@ bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int nc
     const int busy = static_cast<int>(std::min<long long>(per_sm, (ctas + sms - 1) / sms));
     const double warp_cycles = (threads > 256 ? wide : 0.78 * wide) * (rag ? 1.1 : 1.0);  // (the two kernels of cluster_cplx.cuh)
     const double cost = static_cast<double>(rounds) *
-                        (900.0 + 250.0 * std::log2(static_cast<double>(cluster)) + warp_cycles * busy * nw);
+                        (900.0 + 250.0 * std::log2(static_cast<double>(cluster)) + warp_cycles * busy * nw +
+                         1500.0 * ((kCols * n_t + threads - 1) / threads - 1));
     if (best == 0.0 || cost < best) {
       best = cost;
       *p = q;
@@ -83,6 +84,8 @@ bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int nc
   // 41.8 -> 28.3; 120 x 120: 57.2 -> 48.5; 100 x 98: 45.0 -> 42.2.  Clusters of 13 to 16 CTAs
   // fit the chip only seven times (112 of the 152 SMs): 128 x 128, 512 columns: 31.5 -> 30.8, and
   // more of them stay streamed.
+  // Many targets: 64 x 64, 16 columns, M = 200: 256 targets 2.58 -> 0.66, 1024: 2.58 -> 1.52, 4096 would
+  // take 17.8 (streamed 3.0); 128 x 128, 64 columns: 256: 3.66 -> 2.93, 512: 4.52 (streamed 3.80).
   // Ragged periodic sides: 33 x 33, 512 columns: 6.0 -> 1.6; 75 x 90, 1000: 35.2 -> 19.0; 98 x 98: 41.4 ->
   // 36.7; 121 x 119 would take 1.08 of the streamed time, so they are given a margin.
   return best > 0.0 && best * (rag ? 1.15 : 1.0) < 21000.0 + 0.0165 * Lx * Ly * ncols;

@@ -230,7 +230,8 @@ struct CplxClusterArgs {
   int cluster, rows;
 };
 constexpr int kCplxClusterSmem = 227 * 1024 - 3104;  // dynamic shared memory beside the kernel's own
-bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int ncols, ClusterPlan *p, int *clusters);
+bool plan_cluster_cplx(int Lx, int Ly, int px, int py, int nnn, int bond, int ncols, int n_t, ClusterPlan *p,
+                       int *clusters);
 cudaError_t launch_cluster_cplx(CplxClusterArgs a, int bond, const ClusterPlan &p, int clusters, cudaStream_t s);
 
 // Recursion step for the general lattice (complex vectors; nnn: 8 hopping

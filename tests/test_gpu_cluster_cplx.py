@@ -97,16 +97,17 @@ def test_more_targets_than_threads():
     assert max_abs(a11, o11) < TOL and max_abs(a12, o12) < TOL
 
 
-@pytest.mark.parametrize("shape,n", [((180, 180, 1, 1), 4), ((128, 128, 1, 1), 2000)])
-def test_other_calls_stay_streamed(shape, n):
-    """A lattice that does not fit, and more columns of a large one than clusters
-    take in good time."""
+@pytest.mark.parametrize("shape,n,n_t", [((180, 180, 1, 1), 4, 3), ((128, 128, 1, 1), 2000, 3), ((64, 64, 1, 1), 16, 4096)])
+def test_other_calls_stay_streamed(shape, n, n_t):
+    """A lattice that does not fit, and more columns of a large one, or more targets,
+    than clusters take in good time."""
     p = lattice(*shape, -0.3, 1, 8, seed=5)
-    sites = np.random.default_rng(6).choice(p.N, n).astype(np.int32)
+    rng = np.random.default_rng(6)
+    sites, targets = rng.choice(p.N, n).astype(np.int32), rng.choice(p.N, n_t).astype(np.int32)
     lat = gpu_lattice(p, "fp32")
-    a11, a12 = lat.green_moments(sites, sites[:3], 8)
+    a11, a12 = lat.green_moments(sites, targets, 8)
     assert lat.last_tile()[1] > 0
-    o11, o12 = orc.green_moments(as_oracle(p), lat.rescale, sites[:4], sites[:3], 8)
+    o11, o12 = orc.green_moments(as_oracle(p), lat.rescale, sites[:4], targets, 8)
     assert max_abs(a11[:4], o11) < TOL and max_abs(a12[:4], o12) < TOL
 
 
