@@ -302,8 +302,11 @@ Chunks chunks_of(long long rows, int M, int n_E) {
 }  // namespace
 
 // From M = 64 on (64 x 64 outputs: 75 -> 43 us; at M = 32 the FP64 kernel's 39 us stand against
-// 42), to the length at which the 64-bit sums may still hold every digit at its largest.
-bool green_mma_wanted(long long rows, int M, int n_E) { return rows > 0 && n_E > 0 && M >= 64 && M <= (1 << 20); }
+// 42), to the length at which the 64-bit sums may still hold every digit at its largest; not where the
+// digits of the weights outweigh a short sum over few rows (3 rows, 66,000 energies, M = 64: 480 us, 541 here).
+bool green_mma_wanted(long long rows, int M, int n_E) {
+  return rows > 0 && n_E > 0 && M >= 64 && M <= (1 << 20) && (M >= 128 || rows >= 16 || n_E <= 16384);
+}
 
 size_t green_mma_scratch(long long rows, int M, int n_E) {
   const Chunks c = chunks_of(rows, M, n_E);

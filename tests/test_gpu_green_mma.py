@@ -50,9 +50,10 @@ def test_small_rows():
     check(lat, np.array([0, p.N - 1]), targets, 64, np.linspace(-0.9, 0.9, 40) * lat.rescale)
 
 
-@pytest.mark.parametrize("n_s,n_t,n_E", [(600, 230, 2), (1, 3, 66000)])
-def test_more_than_one_set_of_planes(n_s, n_t, n_E):
-    p = wl.random_dwave(16, 64, seed=53)
+@pytest.mark.parametrize("n_s,n_t,M,n_E", [(600, 230, 64, 2), (1, 3, 128, 66000), (1, 3, 64, 17000)])
+def test_more_than_one_set_of_planes(n_s, n_t, M, n_E):
+    """(the last one: the FP64 kernel)"""
+    p = wl.random_dwave(16, M, seed=53)
     rng = np.random.default_rng(1)
     lat = cbdg.Lattice(p, precision="fp32", complex_field=True)
-    check(lat, rng.integers(0, p.N, n_s), rng.integers(0, p.N, n_t), 64, rng.uniform(-0.99, 0.99, n_E) * lat.rescale)
+    check(lat, rng.integers(0, p.N, n_s), rng.integers(0, p.N, n_t), M, rng.uniform(-0.99, 0.99, n_E) * lat.rescale)
