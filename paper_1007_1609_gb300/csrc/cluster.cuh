@@ -587,6 +587,7 @@ int slots_one(const ClusterPlan &p) {
     cudaGetLastError();
     n = 0;
   }
+  if (known.size() >= 4096) known.clear();
   known[key] = n;
   return n;
 }

@@ -38,6 +38,8 @@ int slots_of(const ClusterPlan &p) {
                 : kind == 1 ? cplx_slots_1_0(p)
                 : kind == 2 ? cplx_slots_0_1(p)
                             : cplx_slots_1_1(p);
+  if (n < 1) return n;  // (a failure is not kept)
+  if (known.size() >= 4096) known.clear();
   return known[key] = n;
 }
 
