@@ -120,9 +120,12 @@ __global__ void __launch_bounds__(WIDE ? 384 : kCxNarrow, 1) cluster_cplx_kernel
   if (t == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(nw) : "memory");
   unsigned phase = 0;
   auto arrive = [&]() {
-    __syncwarp();
-    if (CS > 1) cluster_arrive();
-    else if (lane == 0) mbar_arrive(bar);
+    if (CS > 1) {
+      cluster_arrive();
+    } else {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar);
+    }
   };
   auto wait = [&]() {
     if (CS > 1) {
