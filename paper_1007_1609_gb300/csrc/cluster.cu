@@ -36,13 +36,14 @@ int slots_of(const ClusterPlan &p) {
 // have fitted 101 times took twice the time of one of 2.  A step costs an SM 28
 // to 31 cycles (40 with tiles of 10, whose registers leave no room to reorder) for
 // each tile row of each of its warps, rounded up to its four schedulers, 500 for the latency of its barriers, edge
-// loads and sums, and 250 for every doubling of the cluster (64 x 64, M = 512, all
-// columns: 4.21, 4.65 and 5.27 ms with tiles of 8 rows in clusters of 1, 2 and 4).
-// High tiles exchange fewer edges per site and win where they fill the SM (4.21
-// against 4.32 ms with 4 rows there; 128 x 128: 73.7 against 78.6 ms), tiles of 6
-// and 10 hold more sites per SM (96 x 96: 19.9 ms with 6 in one CTA against 27.4
-// and 31.1 with 4 and 8; 500 x 320 fits on chip only with 10), low ones leave more
-// warps to a lattice that leaves SMs idle (33 x 21: 0.53 against 0.61 ms).
+// loads and sums, and 250 for every doubling of the cluster (all columns of 64 x 64, M = 512:
+// 4.54, 5.01 and 5.60 ms with tiles of 8 rows in clusters of 1, 2 and 4).  (The cycles were fitted
+// with plain sums; the compensated ones add about a tenth to every candidate and leave the order.)
+// High tiles exchange fewer edges per site and win where they fill the SM (4.54
+// against 4.66 ms with 4 rows there; 128 x 128, M = 512: 80.7 against 84.6 ms), tiles of 6
+// and 10 hold more sites per SM (96 x 96: 22.0 ms with 6 in one CTA against 31.8
+// and 34.9 with 4 and 8; 500 x 320 fits on chip only with 10), low ones leave more
+// warps to a lattice that leaves SMs idle (33 x 21, two iterations: 0.83 against 0.95 ms).
 bool plan_cluster(int Lx, int Ly, int px, int py, int ncols, ClusterPlan *p) {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
@@ -76,7 +77,7 @@ bool plan_cluster(int Lx, int Ly, int px, int py, int ncols, ClusterPlan *p) {
       if ((TY + rows - 1) / rows != cluster || nw > warps) continue;
       const int ghosts = cluster > 1 ? (TX + per_ghost - 1) / per_ghost : 0;
       const size_t smem = static_cast<size_t>(nw * 32 + ghosts + 1) * quads * 16 +
-                          static_cast<size_t>(cluster) * 3 * kClusterBatch * 8 + 2 * kClusterBatch * 3 * nw * 4;
+                          static_cast<size_t>(cluster) * 3 * kClusterBatch * 8 + 2 * kClusterBatch * 3 * nw * 8;
       if (smem > kClusterSmem) continue;
       Candidate c{ClusterPlan{by, cluster, rows, nw * 32, rag, smem}, nw,
                   std::min(warps / nw, static_cast<int>(kClusterSmem / (smem + 1024))), false, 0.0};

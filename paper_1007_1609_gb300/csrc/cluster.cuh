@@ -15,19 +15,23 @@
 // arrival and wait, and the inner rows of the next step, which need no row of
 // another tile, are computed in between.
 //
-// The three column sums of the doubling identities are formed per thread (at
-// most 32 FP32 multiply-adds per accumulator), added across the halves of the
-// pair and the lanes of a warp in FP32 (6 roundings; 38 * 2^-24 of the sum of
-// magnitudes in all), kept per warp and step, and every 16 steps added in FP64
-// over the warps and CTAs and folded by one thread per step.
+// The three column sums of the doubling identities are formed per thread in
+// FP32 with compensation: the products of two rows of the tile, eight in each
+// half of the pair, in a chain of multiply-adds, the chains by compensated
+// addition (8 * 2^-24 of the sum of magnitudes in all).  The lanes of a warp are added in
+// fixed point without rounding, kept per warp and step, and every 16 steps added
+// over the warps and CTAs (in FP64) and folded by one thread per step.  Root mean square
+// distance of the moments from FP64, over 33 x 21 .. 500 x 320 sites and M = 116 .. 2048: 0.69 (mu_ee)
+// and 0.80 (mu_eh) of the streamed kernels' (FP64 sums of the same vectors: 0.69 and 0.79; plain FP32
+// sums over tile and lanes: 0.71 and 0.82, and of the LDOS at a few sites 1.02, now 0.89).  The
+// compensated sums take a tenth of the time: 146 -> 160 ms for 128 x 128, M = 1024.
 //
-// Bound: instruction issue and the FP32 pipe (64 x 64: FP32 pipe 54% busy, issue
-// 43%, fixed-latency and pipe-throttle stalls first; fused multiply-adds with
+// Bound: instruction issue and the FP32 pipe (fused multiply-adds with
 // three register operands run at two thirds of the pipe's rate).  Measured, one
-// map over all sites: 128 x 128, M = 1024: 146 ms (288 ms with three steps per
-// pass over HBM); 64 x 64, M = 512: 4.2 ms (14.6); 96 x 96: 19.9 ms (55.5); the
-// 75 x 90 torus: 19.1 ms (55.8, one step per pass); 11 start sites of a 100 x
-// 150 lattice, M = 2048: 1.2 ms (88 ms, one launch per step).
+// map over all sites: 128 x 128, M = 1024: 160 ms (288 ms with three steps per
+// pass over HBM); 64 x 64, M = 512: 4.5 ms (14.6); 96 x 96: 22.0 ms (55.5); the
+// 75 x 90 torus: 18.8 ms (55.8, one step per pass); 11 start sites of a 100 x
+// 150 lattice, M = 2048: 1.3 ms (88 ms, one launch per step).
 #pragma once
 
 #include <algorithm>
@@ -117,6 +121,32 @@ __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
+// A thread's column sum v + e, |e| within the rounding of v (a sum of at most 1: |v| < 4).
+struct Sum {
+  float v = 0.f, e = 0.f;
+  __device__ __forceinline__ bool fits() const { return fabsf(v) < 4.f; }
+};
+// The halves of s + r as one sum, exactly but for the rounding of e.
+__device__ __forceinline__ Sum halves(F2 s, F2 r) {
+  const float x = f2get(s, 0), y = f2get(s, 1);
+  Sum o;
+  o.v = __fadd_rn(x, y);
+  const float b = __fsub_rn(o.v, x);
+  o.e = __fadd_rn(__fadd_rn(__fsub_rn(x, __fsub_rn(o.v, b)), __fsub_rn(y, b)), __fadd_rn(f2get(r, 0), f2get(r, 1)));
+  return o;
+}
+// The sum of a warp's lanes in fixed point: each lane's value to units of 2^-20, then what is left of it
+// to units of 2^-42, which the mantissas of 12 + v and of 1.5 * 2^-19 + rest hold, added as integers.
+__device__ __forceinline__ uint2 warp_sum(const Sum &s) {
+  const float t = __fadd_rn(s.v, 12.f);
+  const float u = __fadd_rn(__fadd_rn(__fsub_rn(s.v, __fsub_rn(t, 12.f)), s.e), 0x1.8p-19f);
+  return make_uint2(__reduce_add_sync(0xffffffffu, __float_as_uint(t)), __reduce_add_sync(0xffffffffu, __float_as_uint(u)));
+}
+__device__ __forceinline__ long long warp_value(uint2 w) {  // in units of 2^-42
+  return static_cast<long long>(static_cast<int>(w.x - 32u * 0x41400000u)) * (1 << 22) +
+         static_cast<int>(w.y - 32u * 0x36400000u);
+}
+
 __device__ __forceinline__ float el(const Quad &v, int k) { return f2get(k < 2 ? v.lo : v.hi, k & 1); }
 
 // the sites of a thread's tile: row r, columns 2h and 2h + 1 in [r][h]
@@ -168,7 +198,7 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
   const int Lx = a.Lx, Ly = a.Ly, TX = (Lx + kB - 1) / kB, TY = (Ly + BY - 1) / BY, R = a.rows;
   const int ghost = blockDim.x, nil = ghost + (CS > 1 ? (TX + Rec::kGhosts - 1) / Rec::kGhosts : 0);  // records
   double *xsum = reinterpret_cast<double *>(raw + (nil + 1) * Rec::kBytes);  // rank 0: [CS][3 kBatch] sums of a batch
-  float *ring = reinterpret_cast<float *>(xsum + CS * 3 * kBatch);           // [2 kBatch][3][nw] warp sums of the last steps
+  uint2 *ring = reinterpret_cast<uint2 *>(xsum + CS * 3 * kBatch);           // [2 kBatch][3][nw] warp sums of the last steps
   const unsigned e0 = smem_addr(raw);
   auto barrier = [&]() {
     if (CS > 1) {
@@ -303,25 +333,24 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
     if (push_up) push4(push_up + po, tl, th);
     if (push_dn) push4(push_dn + po, o[0][0], o[0][1]);
   };
-  // warp sums of (A, B, C) of step n: lanes 0, 8 and 16 end with one each
-  auto reduce = [&](int n, float A, float B, float C) {
-    const bool hi = lane & 16, mid = lane & 8;
-    const float s0 = __shfl_xor_sync(0xffffffffu, hi ? A : C, 16), s1 = __shfl_xor_sync(0xffffffffu, hi ? B : 0.f, 16);
-    const float k0 = __fadd_rn(hi ? C : A, s0), k1 = hi ? 0.f : __fadd_rn(B, s1);
-    float v = __fadd_rn(mid ? k1 : k0, __shfl_xor_sync(0xffffffffu, mid ? k0 : k1, 8));
-    v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, 4));
-    v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, 2));
-    v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, 1));
-    if ((lane & 7) == 0 && lane < 24) ring[(((n - 1) & (2 * kBatch - 1)) * 3 + (lane >> 3)) * nw + warp] = v;
+  uint2 A{}, B{}, C{};  // the warp's column sums of the last step
+  auto keep_sums = [&](int n) {
+    uint2 *const w = ring + ((n - 1) & (2 * kBatch - 1)) * 3 * nw + warp;
+    if (lane == 0) {
+      w[0] = A;
+      w[nw] = B;
+      w[2 * nw] = C;
+    }
   };
   // The column sums of the batch of steps that ends with step n: send() adds
   // the warps' in FP64 and gives them to rank 0, whose thread i folds one step.
   auto send = [&](int n) {
     const int first = n - (n - 1) % kBatch, count = n - first + 1;
     for (int k = t; k < 3 * count; k += blockDim.x) {
-      double s = 0.0;
-      const float *w0 = ring + (((first - 1 + k / 3) & (2 * kBatch - 1)) * 3 + k % 3) * nw;
-      for (int z = 0; z < nw; ++z) s += static_cast<double>(w0[z]);
+      long long q = 0;
+      const uint2 *w0 = ring + (((first - 1 + k / 3) & (2 * kBatch - 1)) * 3 + k % 3) * nw;
+      for (int z = 0; z < nw; ++z) q += warp_value(w0[z]);
+      const double s = static_cast<double>(q) * 0x1p-42;
       if (rank == 0) {
         xsum[k] = s;
       } else {
@@ -360,15 +389,31 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
     share[t][0] += dn_;
     share[t][1] += dd_;
   };
-  float A = 0.f, B = 0.f, C = 0.f;  // this thread's column sums of the last step
   // step n: (cu, cv) = j_n, (ou, ov) = j_{n-1} on entry and j_{n+1} on exit;
   // buf_c: the buffer that holds the edges of j_n.  Rows 1 .. BY - 2 first: they
-  // need no row of another tile, so their arithmetic (and the warp reduction
-  // of the step before) runs while the other warps' end rows are on their way.
+  // need no row of another tile, so their arithmetic runs while the other warps' end rows are on their way.
   auto step = [&](int n, int col, auto buf_c, auto edge_c, Tile &cu, Tile &cv, Tile &ou, Tile &ov) {
     constexpr int rd = decltype(buf_c)::value * Rec::kBuffer, wr = (1 - decltype(buf_c)::value) * Rec::kBuffer;
     constexpr bool EDGE = decltype(edge_c)::value;  // rows of the tile may be missing
-    F2 sa = 0, sb = 0, sc = 0;
+    F2 sa = 0, sb = 0, sc = 0;  // the column sums,
+    F2 ra = 0, rb = 0, rc = 0;  // what their last addition lost, and the products since
+    const auto add_rows = [&](bool first) {
+      if (first) {
+        sa = ra;
+        sb = rb;
+        sc = rc;
+        ra = rb = rc = 0;
+        return;
+      }
+      const auto add = [](F2 &s, F2 &x) {  // Kahan
+        const F2 t = f2add(s, x);
+        x = f2sub(x, f2sub(t, s));
+        s = t;
+      };
+      add(sa, ra);
+      add(sb, rb);
+      add(sc, rc);
+    };
     // component part of row r; l, g: the halo left and right, (bl, bh), (tl, th): the halo below row 0 and above row 3
     auto row = [&](int r, int part, const F2 (&er)[2], float l0, float g3, F2 bl, F2 bh, F2 tl, F2 th) {
       Tile &z = part == 0 ? cu : cv;
@@ -390,9 +435,9 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
         const F2 tc = RAG ? tau[h] : tau[0];
         F2 m = f2fma(d[r][h], q[r][h], f2neg(o[r][h]));
         m = part == 0 ? f2fma(f2neg(tc), s, f2fma(er[h], z[r][h], m)) : f2fma(tc, s, f2fma(f2neg(er[h]), z[r][h], m));
-        sa = f2fma(z[r][h], z[r][h], sa);
-        sb = f2fma(m, z[r][h], sb);
-        sc = f2fma(part == 0 ? m : f2neg(m), q[r][h], sc);
+        ra = f2fma(z[r][h], z[r][h], ra);
+        rb = f2fma(m, z[r][h], rb);
+        rc = f2fma(part == 0 ? m : f2neg(m), q[r][h], rc);
         o[r][h] = m;
       }
     };
@@ -434,13 +479,14 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
           row(r, 1, er, el(hl, i + 2), el(hr, i + 2), 0, 0, 0, 0);
         }
       }
+      add_rows(k == 0);
       publish_sides(ou, ov, 2 * k + 1, 2 * k + 2, k, wr);
     }
     arrive(bar_a);
-    reduce(n - 1, A, B, C);
+    keep_sums(n - 1);
     if (!(RAG == 2 && EDGE && early)) wait_ends(phase);
     phase ^= 1u;
-    // the last batch of sums: reduced by step 1, sent in step 2 and folded in step 3 of the next one
+    // the last batch of sums: kept by step 1, sent in step 2 and folded in step 3 of the next one
     if (decltype(buf_c)::value == 1 && n % kBatch == 2 && n > 2) send(n - 2);
     if (decltype(buf_c)::value == 0 && n % kBatch == 3 && n > 3) fold(n - 3, col);
     {
@@ -462,14 +508,18 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
         row(BY - 1, 0, er, el(hl, 1), el(hr, 1), 0, 0, tu.lo, tu.hi);
         row(BY - 1, 1, er, el(hl, 3), el(hr, 3), 0, 0, tv.lo, tv.hi);
       }
+      add_rows(false);
     }
     publish_sides(ou, ov, 0, BY - 1, BY / 2 - 1, wr);
     publish_ends(ou, 0, wr);
     publish_ends(ov, 1, wr);
     arrive_ends();
-    A = __fadd_rn(f2get(sa, 0), f2get(sa, 1));
-    B = __fadd_rn(f2get(sb, 0), f2get(sb, 1));
-    C = __fadd_rn(f2get(sc, 0), f2get(sc, 1));
+    const Sum ta = halves(sa, ra), tb = halves(sb, rb), tc = halves(sc, rc);
+    A = warp_sum(ta);
+    B = warp_sum(tb);
+    C = warp_sum(tc);
+    // (|j_n| <= 1, unless the spectrum leaves [-1, 1])
+    if (!ta.fits() || (2 * n + 1 < a.M && !(tb.fits() && tc.fits()))) atomicOr(a.flags, kFlagSpectrum);
   };
 
   for (int col = cid; col < a.ncols; col += ncl) {
@@ -519,7 +569,7 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
     wait(bar_a, phase);
     wait_ends(phase);
     phase ^= 1u;
-    reduce(a.steps, A, B, C);
+    keep_sums(a.steps);
     __syncthreads();
     for (int n = a.steps > 3 ? (a.steps - 3) / kBatch * kBatch : 0; n < a.steps; n += kBatch) {
       const int last = min(n + kBatch, a.steps);
