@@ -95,7 +95,7 @@ bool plan_adjoint_cluster(int Lx, int Ly, int px, int py, int ncols, int M, Clus
     }
   }
   if (best == 0.0) return false;
-  const size_t lanes = static_cast<size_t>(*clusters) * p->cluster * p->threads;
+  const size_t lanes = static_cast<size_t>(p->cluster) * p->threads;
   *ck_bytes = lanes * ((M - 2) / kSegment + 1) * 16 * sizeof(float4);
   *acc_bytes = lanes * 64 * sizeof(float2);
   return true;

@@ -1122,6 +1122,34 @@ cbdg_status order_parameter_impl(cbdg_lattice *L, double T, int kernel, double l
   return run_columns(L, L->sites_all.as<int32_t>(), L->N, M, nullptr, nullptr, 1, true);
 }
 
+// Allocates the scratch of the on-chip adjoint, ck and acc bytes a cluster, for as many of *clusters as
+// the workspace cap or, without one, half of the free memory holds (as the streamed adjoint sizes its
+// chunks).  *clusters = 0: less than half of them fit, or the allocation failed; the streamed
+// adjoint takes what there is.
+cbdg_status adjoint_scratch(cbdg_lattice *L, size_t ck, size_t acc, int *clusters) {
+  const size_t held = L->adj_ck.bytes + L->adj_part.bytes;
+  if (L->adj_ck.bytes < *clusters * ck || L->adj_part.bytes < *clusters * acc || L->ws_mb > 0) {
+    size_t cap = static_cast<size_t>(L->ws_mb) << 20;
+    if (L->ws_mb == 0) {
+      size_t fr = 0, tot = 0;
+      CK(cudaMemGetInfo(&fr, &tot));
+      cap = (fr + held) / 2;
+    }
+    const size_t n = cap / (ck + acc);
+    if (n < static_cast<size_t>(*clusters)) *clusters = 2 * n >= static_cast<size_t>(*clusters) ? static_cast<int>(n) : 0;
+  }
+  if (*clusters == 0) return CBDG_OK;
+  cudaError_t e = L->adj_ck.ensure(*clusters * ck);
+  if (e == cudaSuccess) e = L->adj_part.ensure(*clusters * acc);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    *clusters = 0;
+    return CBDG_OK;
+  }
+  CK(e);
+  return CBDG_OK;
+}
+
 // One adjoint run of the self-consistency map with the weights w_i = dL/dDelta_out,i
 // already in L->adj_w (device): leaves dL/deps, dL/dDelta_in and dL/dt in
 // L->adj_out ([N] eps, [N] Delta, [N*4] hop).
@@ -1145,13 +1173,16 @@ cbdg_status adjoint_run(cbdg_lattice *L, double T, int M, const int32_t *cols = 
   {
     ClusterPlan plan;
     int clusters = 0;
-    size_t ck_bytes = 0, acc_bytes = 0;
-    if (on_chip(L) &&
-        plan_adjoint_cluster(L->Lx, L->Ly, L->px, L->py, n_cols, M, &plan, &clusters, &ck_bytes, &acc_bytes) &&
-        (L->ws_mb == 0 || ck_bytes + acc_bytes <= static_cast<size_t>(L->ws_mb) << 20)) {
-      CK(L->adj_ck.ensure(ck_bytes));
-      CK(L->adj_part.ensure(acc_bytes));
-      CK(cudaMemsetAsync(L->adj_part.p, 0, acc_bytes, L->stream));
+    size_t ck_bytes = 0, acc_bytes = 0;  // scratch of a cluster
+    bool fits = on_chip(L) && plan_adjoint_cluster(L->Lx, L->Ly, L->px, L->py, n_cols, M, &plan, &clusters, &ck_bytes,
+                                                   &acc_bytes);
+    if (fits) {
+      st = adjoint_scratch(L, ck_bytes, acc_bytes, &clusters);
+      if (st != CBDG_OK) return st;
+      fits = clusters > 0;
+    }
+    if (fits) {
+      CK(cudaMemsetAsync(L->adj_part.p, 0, clusters * acc_bytes, L->stream));
       CK(L->adj_out.ensure(static_cast<size_t>(N) * 6 * sizeof(double)));
       AdjointClusterArgs c{};
       c.params = L->params.as<float>();

@@ -199,7 +199,7 @@ struct AdjointClusterArgs {
   int cluster, rows;
 };
 // Plans the launch for ncols columns and M moments; false where the lattice or M
-// does not fit.  clusters: how many run; ck_bytes and acc_bytes: their scratch.
+// does not fit.  clusters: how many run; ck_bytes and acc_bytes: the scratch of one.
 bool plan_adjoint_cluster(int Lx, int Ly, int px, int py, int ncols, int M, ClusterPlan *p, int *clusters,
                           size_t *ck_bytes, size_t *acc_bytes);
 cudaError_t launch_adjoint_cluster(AdjointClusterArgs a, const ClusterPlan &p, int clusters, cudaStream_t s);
