@@ -233,9 +233,8 @@ cbdg_status cbdg_scf_step(cbdg_lattice *lat, double T, int32_t M, double mix,
  * Any output may be NULL; outputs are host or device arrays.  Real lattices
  * run the real recursion (imaginary parts 0), general ones complex vectors.
  * FP32 lattices with one real hopping run it in the registers of thread-block
- * clusters where they fit (M <= 4096, periodic sides multiples of four): pairs
- * (j_n, j_{n+1}) are kept every 8 steps and the recursion is run backwards
- * between them.  Elsewhere the forward recursion runs without doubling, keeps
+ * clusters where they fit (M <= 4096, periodic sides multiples of four, memory for
+ * the vectors j_n of a start site per cluster).  Elsewhere the forward recursion runs without doubling, keeps
  * checkpoints of (j_{kS}, j_{kS+1}) every S = ceil(sqrt(M)) steps and recomputes
  * each segment during the reverse sweep
  *   lam_m = y_m + 2 H~ lam_{m+1} - lam_{m+2},

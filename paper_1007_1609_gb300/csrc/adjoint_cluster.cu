@@ -17,7 +17,7 @@ cudaError_t adjoint_launch_1(const AdjointClusterArgs &a, const ClusterPlan &p, 
 
 namespace {
 
-constexpr int kQuads = 41, kGhosts = 2, kSegment = 8;  // as in adjoint_cluster.cuh
+constexpr int kQuads = 41, kGhosts = 2;  // as in adjoint_cluster.cuh
 constexpr int kMaxM = 4096;                             // the column's source table is in shared memory
 
 int slots_of(const ClusterPlan &p) {
@@ -96,7 +96,7 @@ bool plan_adjoint_cluster(int Lx, int Ly, int px, int py, int ncols, int M, Clus
   }
   if (best == 0.0) return false;
   const size_t lanes = static_cast<size_t>(p->cluster) * p->threads;
-  *ck_bytes = lanes * ((M - 2) / kSegment + 1) * 16 * sizeof(float4);
+  *ck_bytes = lanes * (M - 1) * 8 * sizeof(float4);
   *acc_bytes = lanes * 64 * sizeof(float2);
   return true;
 }
@@ -104,7 +104,6 @@ bool plan_adjoint_cluster(int Lx, int Ly, int px, int py, int ncols, int M, Clus
 cudaError_t launch_adjoint_cluster(AdjointClusterArgs a, const ClusterPlan &p, int clusters, cudaStream_t s) {
   a.cluster = p.cluster;
   a.rows = p.rows;
-  a.n_ck = (a.M - 2) / kSegment + 1;
   return p.rag ? adjoint_launch_1(a, p, clusters, s) : adjoint_launch_0(a, p, clusters, s);
 }
 

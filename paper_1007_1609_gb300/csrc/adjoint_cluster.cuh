@@ -3,27 +3,32 @@
 // FP32 vectors; a periodic side a multiple of 4).
 //
 // A cluster takes one start site at a time through the forward recursion and
-// back.  On the way back the vectors j_m are not read from memory: the recursion
-// runs in reverse, j_{m-2} = 2 H~ j_{m-1} - j_m, beside lam_{m-1} = y_{m-1} + 2 H~ lam_m -
-// lam_{m+1}, so one pass over the tile's edges serves both and the gradient sums,
-// which need lam_m and j_{m-1} at a site and at its right and upper neighbours.
-// Every kSegment steps (j_{kS}, j_{kS+1}) are replaced by the pair that the forward
-// pass left in a scratch of the cluster.  Run back over all 512 steps the pair
-// would carry two to four times the forward rounding; the gradient's distance
-// from FP64 (64 x 64, M = 512; stored vectors: 0.95, 1.0 and 0.4e-7 in eps, t and
-// Delta) and the time are 1.6, 1.6 and 0.6e-7 at 30.0 ms with 32 steps, 1.1, 1.3
-// and 0.4e-7 at 35 ms with 8 and no less at 39 ms with 4.
+// back.  The forward pass leaves every j_n in a scratch of the cluster (32 floats a thread
+// and step, written past the caches' working set), the way back fetches them again, each
+// thread what it wrote itself: j_{m-2} is on its way while step m forms lam_{m-1} = y_{m-1} +
+// 2 H~ lam_m - lam_{m+1} and the gradient sums, which need lam_m and j_{m-1} at a site and at
+// its right and upper neighbours.  (Running the recursion backwards between pairs kept every
+// 8 steps takes a quarter of the scratch and adds the rounding of the reversed steps: table below.)
 //
 // The layout is cluster.cuh's with tiles of 4 x 4: a thread holds the four
-// vectors (128 registers) and 64 gradient sums of its sites.  The sums are plain
-// FP32 over kFlush steps of one column and then added to compensated pairs (an FP32
-// head and the exact rounding errors) in a scratch of the CTA, which the final
-// kernel adds over the clusters in FP64.
+// vectors (128 registers) and 64 gradient sums of its sites.  The products of a step are
+// added first, then to FP32 sums over kFlush steps of one column, those to compensated
+// pairs (an FP32 head and the exact rounding errors) in a scratch of the CTA, and the final
+// kernel adds the pairs over the clusters in FP64.
 //
-// Bound: the FP32 pipe and instruction issue, 36 multiply-adds per site and step
-// on the way back and 12 on the way there.  64 x 64, M = 512: 101 ms with the
-// vectors in HBM (forward, recomputation and reverse three steps per pass,
-// sums in launches of their own) -> 35 ms.
+// Distance of the gradient from FP64, root mean square relative to the streamed adjoint's
+// (columns added with compensation, steps in FP64), geometric mean over 24 gradients of 16^2 .. 64^2 sites,
+// M = 77 .. 512, in eps, t and Delta, and the time of 64 x 64, M = 512:
+//   reversed between pairs every 8 steps, products added one by one:  0.97 1.05 0.93   35.2 ms
+//   the same, every sum in FP64:                                      0.92 0.96 0.89
+//   stored vectors, products of a step first (this):                  0.91 0.93 0.84   37.2 ms
+//   with kFlush 32 or 16 in place of 64:                              0.92 0.94 0.84   40.2, 45.6 ms
+//   stored vectors, every sum in FP64:                                0.86 0.86 0.79
+//
+// Bound: the FP32 pipe and instruction issue, 24 multiply-adds per site and step
+// on the way back and 12 on the way there, beside 69 GB written and as much read (64 x 64, M = 512).
+// That call took 101 ms with one launch per step (forward, recomputation and reverse three
+// steps per pass, sums in launches of their own).
 #pragma once
 
 #include "cluster.cuh"
@@ -31,7 +36,6 @@
 namespace cbdg {
 namespace {
 
-constexpr int kSegment = 8;  // steps between the pairs kept by the forward pass
 constexpr int kFlush = 64;   // steps between two moves of the sums to the scratch
 // A thread's record in shared memory, in quads: twice (double buffer) the edges
 // of j and of lam (Record<4>'s eight quads each), then its rows of 2 (eps - mu) / a
@@ -72,20 +76,20 @@ __device__ __forceinline__ void grad_row(GradSums &g, int r, const Tile4 &lu, co
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const F2 a = lu[r][h], b = lv[r][h], c = ju[r][h], e = jv[r][h];
-    g.e[r][h] = f2fma(a, c, f2fma(f2neg(b), e, g.e[r][h]));
-    g.d[r][h] = f2fma(a, e, f2fma(b, c, g.d[r][h]));
+    g.e[r][h] = f2add(g.e[r][h], f2fma(a, c, f2fma(f2neg(b), e, 0)));
+    g.d[r][h] = f2add(g.d[r][h], f2fma(a, e, f2fma(b, c, 0)));
     const F2 a1 = r < 3 ? lu[r < 3 ? r + 1 : r][h] : (h ? tlu.hi : tlu.lo);
     const F2 b1 = r < 3 ? lv[r < 3 ? r + 1 : r][h] : (h ? tlv.hi : tlv.lo);
     const F2 c1 = r < 3 ? ju[r < 3 ? r + 1 : r][h] : (h ? tju.hi : tju.lo);
     const F2 e1 = r < 3 ? jv[r < 3 ? r + 1 : r][h] : (h ? tjv.hi : tjv.lo);
-    g.y[r][h] = f2fma(f2neg(a), c1, f2fma(f2neg(a1), c, f2fma(b, e1, f2fma(b1, e, g.y[r][h]))));
+    g.y[r][h] = f2add(g.y[r][h], f2fma(f2neg(a), c1, f2fma(f2neg(a1), c, f2fma(b, e1, f2fma(b1, e, 0)))));
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const float a = at(lu, r, k), b = at(lv, r, k), c = at(ju, r, k), e = at(jv, r, k);
     const float a1 = k < 3 ? at(lu, r, k < 3 ? k + 1 : k) : rlu, b1 = k < 3 ? at(lv, r, k < 3 ? k + 1 : k) : rlv;
     const float c1 = k < 3 ? at(ju, r, k < 3 ? k + 1 : k) : rju, e1 = k < 3 ? at(jv, r, k < 3 ? k + 1 : k) : rjv;
-    g.x[r][k] = __fmaf_rn(-a, c1, __fmaf_rn(-a1, c, __fmaf_rn(b, e1, __fmaf_rn(b1, e, g.x[r][k]))));
+    g.x[r][k] = __fadd_rn(g.x[r][k], __fmaf_rn(-a, c1, __fmaf_rn(-a1, c, __fmaf_rn(b, e1, __fmul_rn(b1, e)))));
   }
 }
 
@@ -206,7 +210,7 @@ __global__ void __launch_bounds__(256, 1) adjoint_cluster_kernel(AdjointClusterA
     }
   };
   auto live = [&](int r) { return !RAG || r < rl; };
-  float4 *const ck = a.ck + static_cast<size_t>(blockIdx.x) * a.n_ck * 16 * blockDim.x + t;
+  float4 *const ck = a.ck + static_cast<size_t>(blockIdx.x) * (a.M - 1) * 8 * blockDim.x + t;
   float2 *const acc = a.acc + static_cast<size_t>(blockIdx.x) * 64 * blockDim.x + t;
 
   // forward: (cu, cv) = j_n, (ou, ov) = j_{n-1} -> j_{n+1}
@@ -247,23 +251,24 @@ __global__ void __launch_bounds__(256, 1) adjoint_cluster_kernel(AdjointClusterA
     publish_ends(ou, ov, 0, wr);
     arrive_ends();
   };
-  // rows [ra, rb] of a pair kept by the forward pass: vector v (0: j_{kS}, 1: j_{kS+1})
-  auto keep = [&](int k, int v, const Tile4 &u, const Tile4 &w) {
+  // j_n to and from the cluster's scratch; a thread reads what it wrote itself
+  auto keep = [&](int n, const Tile4 &u, const Tile4 &v) {
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      ck[(static_cast<size_t>(k) * 16 + v * 8 + r) * blockDim.x] =
-          make_float4(at(u, r, 0), at(u, r, 1), at(u, r, 2), at(u, r, 3));
-      ck[(static_cast<size_t>(k) * 16 + v * 8 + 4 + r) * blockDim.x] =
-          make_float4(at(w, r, 0), at(w, r, 1), at(w, r, 2), at(w, r, 3));
+      __stcs(ck + (static_cast<size_t>(n) * 8 + r) * blockDim.x, make_float4(at(u, r, 0), at(u, r, 1), at(u, r, 2), at(u, r, 3)));
+      __stcs(ck + (static_cast<size_t>(n) * 8 + 4 + r) * blockDim.x, make_float4(at(v, r, 0), at(v, r, 1), at(v, r, 2), at(v, r, 3)));
     }
   };
-  auto fetch_row = [&](int k, int v, int r, Tile4 &u, Tile4 &w) {
-    const float4 p = ck[(static_cast<size_t>(k) * 16 + v * 8 + r) * blockDim.x];
-    const float4 q = ck[(static_cast<size_t>(k) * 16 + v * 8 + 4 + r) * blockDim.x];
-    u[r][0] = f2pack(p.x, p.y);
-    u[r][1] = f2pack(p.z, p.w);
-    w[r][0] = f2pack(q.x, q.y);
-    w[r][1] = f2pack(q.z, q.w);
+  auto fetch = [&](int n, Tile4 &u, Tile4 &v) {
+#pragma unroll
+    for (int r : {1, 2, 0, 3}) {
+      const float4 p = __ldcs(ck + (static_cast<size_t>(n) * 8 + r) * blockDim.x);
+      const float4 q = __ldcs(ck + (static_cast<size_t>(n) * 8 + 4 + r) * blockDim.x);
+      u[r][0] = f2pack(p.x, p.y);
+      u[r][1] = f2pack(p.z, p.w);
+      v[r][0] = f2pack(q.x, q.y);
+      v[r][1] = f2pack(q.z, q.w);
+    }
   };
 
   for (int col = cid; col < a.ncols; col += ncl) {
@@ -292,7 +297,7 @@ __global__ void __launch_bounds__(256, 1) adjoint_cluster_kernel(AdjointClusterA
         put(z, r2, c, sr == r2 && sc == c ? v : at(z, r2, c));
       }
     };
-    Tile4 pu, pv, qu, qv;  // j_{n-1}, j_n, later j_{m-1}, j_m
+    Tile4 pu, pv, qu, qv;  // j_{n-1}, j_n, later j_{m-1}, j_{m-2}
     {
       const double am = a.scal[kScalA];
       const float m1 = static_cast<float>((a.eps[site] - a.mu) / am), dl = static_cast<float>(a.delta[site].x / am);
@@ -317,40 +322,30 @@ __global__ void __launch_bounds__(256, 1) adjoint_cluster_kernel(AdjointClusterA
     publish_sides(qu, qv, 0, 3, 1, 0, 0);
     publish_ends(qu, qv, 0, 0);
     arrive_ends();
-    keep(0, 0, pu, pv);
-    keep(0, 1, qu, qv);
-    for (int n = 1; n <= a.M - 2;) {
+    keep(0, pu, pv);
+    if (a.M > 2) keep(1, qu, qv);
+    // up to j_{M-2}, the last one that the sums read
+    for (int n = 1; n <= a.M - 3;) {
       forward(std::integral_constant<int, 0>{}, qu, qv, pu, pv);
-      if (n % kSegment == 0) {
-        keep(n / kSegment, 0, qu, qv);
-        keep(n / kSegment, 1, pu, pv);
-      }
-      if (++n > a.M - 2) break;
+      keep(++n, pu, pv);
+      if (n > a.M - 3) break;
       forward(std::integral_constant<int, 1>{}, pu, pv, qu, qv);
-      if (n % kSegment == 0) {
-        keep(n / kSegment, 0, pu, pv);
-        keep(n / kSegment, 1, qu, qv);
-      }
-      ++n;
+      keep(++n, qu, qv);
     }
-    if (a.M & 1) {  // an odd number of steps: (p, q) = (j_{M-1}, j_{M-2})
+    if (a.M & 1) {  // (p) = j_{M-2}
 #pragma unroll
       for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          F2 x = pu[r][h];
           pu[r][h] = qu[r][h];
-          qu[r][h] = x;
-          x = pv[r][h];
           pv[r][h] = qv[r][h];
-          qv[r][h] = x;
         }
     }
     wait(bar_a, phase);
     wait_ends(phase);
     phase ^= 1u;
     __syncthreads();  // tab
-    // back: (p) = j_{m-1}, (q) = j_m, (l) = lam_m, (k) = lam_{m+1}, m = M - 1
+    // back: (p) = j_{m-1}, (l) = lam_m, (k) = lam_{m+1}, m = M - 1
     Tile4 lu, lv, ku, kv;
     GradSums g;
 #pragma unroll
@@ -371,33 +366,26 @@ __global__ void __launch_bounds__(256, 1) adjoint_cluster_kernel(AdjointClusterA
     publish_ends(pu, pv, 0, 0);
     publish_ends(lu, lv, 1, 0);
     arrive_ends();
-    // step m: sums of lam_m and j_{m-1}; (jo) = j_m -> j_{m-2}, (ko) = lam_{m+1} -> lam_{m-1} (m > 1)
+    // step m: sums of lam_m and (j) = j_{m-1}; (o) = j_{m-2}, (w) = lam_{m+1} -> lam_{m-1} (m > 1)
     auto back = [&](int m, auto buf_c, Tile4 &ju, Tile4 &jv, Tile4 &ou, Tile4 &ov, Tile4 &zu, Tile4 &zv, Tile4 &wu,
                     Tile4 &wv) {
       constexpr int rd = decltype(buf_c)::value * kAdjBuffer * 16, wr = (1 - decltype(buf_c)::value) * kAdjBuffer * 16;
       constexpr int fl = kAdjField * 16;  // lam's edges
-      const bool fresh = m >= 2 && (m - 2) % kSegment == 0;  // j_{m-2}, j_{m-1} were kept
-      const int k = (m - 2) / kSegment;
       const Quad none{0, 0};
       F2 er[2], dr[2];
+      if (m >= 2) fetch(m - 2, ou, ov);  // on its way during the step
       wait(bar_a, phase);
       {
-        const Quad hl = lds4(lf + rd), hr = lds4(rt + rd), ll = lds4(lf + rd + fl), lr = lds4(rt + rd + fl);
+        const Quad hr = lds4(rt + rd), ll = lds4(lf + rd + fl), lr = lds4(rt + rd + fl);
 #pragma unroll
         for (int r = 1; r < 3; ++r)
           if (live(r)) {
             grad_row(g, r, zu, zv, ju, jv, el(lr, r - 1), el(lr, r + 1), el(hr, r - 1), el(hr, r + 1), none, none, none,
                      none);
             params(r, er, dr);
-            stencil_row<0>(ju, jv, ou, r, er, dr, tau, el(hl, r - 1), el(hr, r - 1), 0, 0, 0, 0);
-            stencil_row<1>(jv, ju, ov, r, er, dr, tau, el(hl, r + 1), el(hr, r + 1), 0, 0, 0, 0);
             stencil_row<0>(zu, zv, wu, r, er, dr, tau, el(ll, r - 1), el(lr, r - 1), 0, 0, 0, 0);
             stencil_row<1>(zv, zu, wv, r, er, dr, tau, el(ll, r + 1), el(lr, r + 1), 0, 0, 0, 0);
           }
-      }
-      if (fresh) {
-        fetch_row(k, 0, 1, ou, ov);
-        fetch_row(k, 0, 2, ou, ov);
       }
       add_source(m - 1, 1, 2, a.part ? wv : wu);
       publish_sides(ou, ov, 1, 2, 0, 0, wr);
@@ -406,14 +394,10 @@ __global__ void __launch_bounds__(256, 1) adjoint_cluster_kernel(AdjointClusterA
       wait_ends(phase);
       phase ^= 1u;
       {
-        const Quad hl = lds4(lf + rd + 16), hr = lds4(rt + rd + 16);
-        const Quad ll = lds4(lf + rd + fl + 16), lr = lds4(rt + rd + fl + 16);
+        const Quad hr = lds4(rt + rd + 16), ll = lds4(lf + rd + fl + 16), lr = lds4(rt + rd + fl + 16);
         if (live(0)) {
           grad_row(g, 0, zu, zv, ju, jv, el(lr, 0), el(lr, 2), el(hr, 0), el(hr, 2), none, none, none, none);
           params(0, er, dr);
-          const Quad bu = lds4(dn + rd), bv = lds4(dn + rd + 16);
-          stencil_row<0>(ju, jv, ou, 0, er, dr, tau, el(hl, 0), el(hr, 0), bu.lo, bu.hi, 0, 0);
-          stencil_row<1>(jv, ju, ov, 0, er, dr, tau, el(hl, 2), el(hr, 2), bv.lo, bv.hi, 0, 0);
           const Quad cu = lds4(dn + rd + fl), cv = lds4(dn + rd + fl + 16);
           stencil_row<0>(zu, zv, wu, 0, er, dr, tau, el(ll, 0), el(lr, 0), cu.lo, cu.hi, 0, 0);
           stencil_row<1>(zv, zu, wv, 0, er, dr, tau, el(ll, 2), el(lr, 2), cv.lo, cv.hi, 0, 0);
@@ -422,17 +406,9 @@ __global__ void __launch_bounds__(256, 1) adjoint_cluster_kernel(AdjointClusterA
           const Quad tu = lds4(up + rd), tv = lds4(up + rd + 16), su = lds4(up + rd + fl), sv = lds4(up + rd + fl + 16);
           grad_row(g, 3, zu, zv, ju, jv, el(lr, 1), el(lr, 3), el(hr, 1), el(hr, 3), su, sv, tu, tv);
           params(3, er, dr);
-          stencil_row<0>(ju, jv, ou, 3, er, dr, tau, el(hl, 1), el(hr, 1), 0, 0, tu.lo, tu.hi);
-          stencil_row<1>(jv, ju, ov, 3, er, dr, tau, el(hl, 3), el(hr, 3), 0, 0, tv.lo, tv.hi);
           stencil_row<0>(zu, zv, wu, 3, er, dr, tau, el(ll, 1), el(lr, 1), 0, 0, su.lo, su.hi);
           stencil_row<1>(zv, zu, wv, 3, er, dr, tau, el(ll, 3), el(lr, 3), 0, 0, sv.lo, sv.hi);
         }
-      }
-      if (fresh) {
-        fetch_row(k, 0, 0, ou, ov);
-        fetch_row(k, 0, 3, ou, ov);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) fetch_row(k, 1, r, ju, jv);
       }
       add_source(m - 1, 0, 3, a.part ? wv : wu);
       publish_sides(ou, ov, 0, 3, 1, 0, wr);

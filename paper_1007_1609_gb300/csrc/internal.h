@@ -190,11 +190,11 @@ struct AdjointClusterArgs {
   const double2 *delta;
   const int32_t *sites;    // [ncols]
   const double *w, *u, *tab;
-  float4 *ck;              // [CTAs][n_ck][16][threads] kept pairs
+  float4 *ck;              // [CTAs][M - 1][8][threads] the vectors j_0 .. j_{M-2} of a column
   float2 *acc;             // [CTAs][64][threads] gradient sums, zero before the first launch
   unsigned int *flags;
   double mu, hop, scale;
-  int stride, part, n_ck;
+  int stride, part;
   int Lx, Ly, px, py, ncols, M;
   int cluster, rows;
 };
