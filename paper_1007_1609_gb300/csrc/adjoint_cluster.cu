@@ -2,11 +2,10 @@
 // adjoint (adjoint_cluster.cuh).
 #include <algorithm>
 #include <cmath>
-#include <map>
-#include <mutex>
 #include <tuple>
 
 #include "internal.h"
+#include "slot_table.h"
 
 namespace cbdg {
 
@@ -21,15 +20,11 @@ constexpr int kQuads = 41, kGhosts = 2;  // as in adjoint_cluster.cuh
 constexpr int kMaxM = 4096;                             // the column's source table is in shared memory
 
 int slots_of(const ClusterPlan &p) {
-  static std::mutex mutex;
-  static std::map<std::tuple<int, int, int, int, size_t>, int> known;
+  static SlotTable<std::tuple<int, int, int, int, size_t>> known;
   int dev = 0;
   cudaGetDevice(&dev);
-  std::lock_guard<std::mutex> lock(mutex);
-  const auto key = std::make_tuple(dev, p.rag, p.cluster, p.threads, p.smem);
-  const auto it = known.find(key);
-  if (it != known.end()) return it->second;
-  return known[key] = p.rag ? adjoint_slots_1(p) : adjoint_slots_0(p);
+  return known.get(std::make_tuple(dev, p.rag, p.cluster, p.threads, p.smem),
+                   [&] { return p.rag ? adjoint_slots_1(p) : adjoint_slots_0(p); });
 }
 
 // Sums over the clusters (heads and tails in FP64); one thread per site.

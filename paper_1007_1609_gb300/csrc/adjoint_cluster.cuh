@@ -467,7 +467,7 @@ int adjoint_slots_one(const ClusterPlan &p) {
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k, &l.cfg);
   if (e != cudaSuccess) {
     cudaGetLastError();
-    return 0;
+    return -1;
   }
   return n;
 }

@@ -35,13 +35,12 @@
 #pragma once
 
 #include <algorithm>
-#include <map>
-#include <mutex>
 #include <tuple>
 #include <type_traits>
 
 #include "f32x2.cuh"
 #include "internal.h"
+#include "slot_table.h"
 
 namespace cbdg {
 namespace {
@@ -624,30 +623,25 @@ struct Launch {
   }
 };
 
-// Clusters of the plan's shape that the current device holds at once (0: none).
+// Clusters of the plan's shape that the current device holds at once (0: none; negative: the query failed).
 template <int BY, int RAG>
 int slots_one(const ClusterPlan &p) {
-  static std::mutex mutex;
-  static std::map<std::tuple<int, int, int, size_t>, int> known;  // by device, cluster, CTA size and shared memory
+  static SlotTable<std::tuple<int, int, int, size_t>> known;  // by device, cluster, CTA size and shared memory
   int dev = 0;
   cudaGetDevice(&dev);
-  std::lock_guard<std::mutex> lock(mutex);
-  const auto key = std::make_tuple(dev, p.cluster, p.threads, p.smem);
-  const auto it = known.find(key);
-  if (it != known.end()) return it->second;
-  auto k = cluster_kernel<BY, RAG>;
-  Launch<BY, RAG> l(p);
-  int n = 0;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kClusterSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k, &l.cfg);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    n = 0;
-  }
-  if (known.size() >= 4096) known.clear();
-  known[key] = n;
-  return n;
+  return known.get(std::make_tuple(dev, p.cluster, p.threads, p.smem), [&] {
+    auto k = cluster_kernel<BY, RAG>;
+    Launch<BY, RAG> l(p);
+    int n = 0;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kClusterSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k, &l.cfg);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return -1;
+    }
+    return n;
+  });
 }
 
 template <int BY, int RAG>

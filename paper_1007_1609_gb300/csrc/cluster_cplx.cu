@@ -2,11 +2,10 @@
 // general lattices (cluster_cplx.cuh).
 #include <algorithm>
 #include <cmath>
-#include <map>
-#include <mutex>
 #include <tuple>
 
 #include "internal.h"
+#include "slot_table.h"
 
 namespace cbdg {
 
@@ -25,22 +24,16 @@ constexpr int kRecord = 33, kCols = 2, kMaxThreads = 384;  // as in cluster_cplx
 
 // p.rag: nnn + 2 bond + 4 for periodic sides that the tiles do not divide
 int slots_of(const ClusterPlan &p) {
-  static std::mutex mutex;
-  static std::map<std::tuple<int, int, int, int, size_t>, int> known;
+  static SlotTable<std::tuple<int, int, int, int, size_t>> known;
   int dev = 0;
   cudaGetDevice(&dev);
-  std::lock_guard<std::mutex> lock(mutex);
-  const auto key = std::make_tuple(dev, p.rag, p.cluster, p.threads, p.smem);
-  const auto it = known.find(key);
-  if (it != known.end()) return it->second;
-  const int kind = p.rag & 3;
-  const int n = kind == 0   ? cplx_slots_0_0(p)
-                : kind == 1 ? cplx_slots_1_0(p)
-                : kind == 2 ? cplx_slots_0_1(p)
-                            : cplx_slots_1_1(p);
-  if (n < 1) return n;  // (a failure is not kept)
-  if (known.size() >= 4096) known.clear();
-  return known[key] = n;
+  return known.get(std::make_tuple(dev, p.rag, p.cluster, p.threads, p.smem), [&] {
+    const int kind = p.rag & 3;
+    return kind == 0   ? cplx_slots_0_0(p)
+           : kind == 1 ? cplx_slots_1_0(p)
+           : kind == 2 ? cplx_slots_0_1(p)
+                       : cplx_slots_1_1(p);
+  });
 }
 
 }  // namespace

@@ -536,7 +536,7 @@ int cplx_slots_one(const ClusterPlan &p) {
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k, &l.cfg);
   if (e != cudaSuccess) {
     cudaGetLastError();
-    return 0;
+    return -1;
   }
   return n;
 }
