@@ -359,7 +359,8 @@ enum {
                                     rescale (frozen a, e.g. for finite differences);
                                     0 = Gershgorin (default) */
   CBDG_OPT_WAIT_LIMIT_MS = 9,    /* limit of every wait of the recursion kernels on a staged
-                                    copy (default 2000); on expiry the call returns
+                                    copy or, on chip, on the other warps of a CTA
+                                    (default 2000); on expiry the call returns
                                     CBDG_ERR_CUDA and the lattice stays usable */
   CBDG_OPT_TEST_STALL_COPY = 10, /* test hook for failure detection: 1 makes the first staged
                                     row of each recursion CTA wait for 16 bytes that never

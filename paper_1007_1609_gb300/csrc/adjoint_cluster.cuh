@@ -125,10 +125,7 @@ __global__ void __launch_bounds__(256, 1) adjoint_cluster_kernel(AdjointClusterA
     if (mbar_try(bar, parity)) return;
     const unsigned long long t0 = global_ns();
     for (unsigned it = 0; !mbar_try(bar, parity); ++it)
-      if ((it & 255u) == 255u && global_ns() - t0 > kWaitNs) {
-        atomicOr(a.flags, kFlagTimeout);
-        break;
-      }
+      if ((it & 255u) == 255u && expired(t0, a.wait_ns, a.flags)) break;
   };
   auto arrive_ends = [&]() {
     if (CS > 1) cluster_arrive();

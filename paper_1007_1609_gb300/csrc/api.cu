@@ -471,6 +471,7 @@ cbdg_status run_cplx_on_chip(cbdg_lattice *L, const void *params, const int32_t 
   c.delta = L->delta.as<double2>();
   c.sites = sites;
   c.flags = L->flags.as<unsigned int>();
+  c.wait_ns = static_cast<unsigned long long>(L->wait_ms) * 1000000ull;
   c.mu = L->mu;
   c.tol = tol;
   c.n_dirs = L->n_dirs;
@@ -545,6 +546,7 @@ cbdg_status run_columns(cbdg_lattice *L, const int32_t *sites, int n_sites, int 
     c.mu_ee = mom_ee;
     c.mu_eh = mom_eh;
     c.flags = L->flags.as<unsigned int>();
+    c.wait_ns = static_cast<unsigned long long>(L->wait_ms) * 1000000ull;
     c.mu = L->mu;
     c.hop = L->hop_all;
     c.tol = 1e-4;
@@ -1193,6 +1195,7 @@ cbdg_status adjoint_run(cbdg_lattice *L, double T, int M, const int32_t *cols = 
       c.ck = L->adj_ck.as<float4>();
       c.acc = L->adj_part.as<float2>();
       c.flags = L->flags.as<unsigned int>();
+      c.wait_ns = static_cast<unsigned long long>(L->wait_ms) * 1000000ull;
       c.mu = L->mu;
       c.hop = L->hop_all;
       c.Lx = L->Lx;

@@ -46,7 +46,6 @@ namespace cbdg {
 namespace {
 
 constexpr int kB = 4;           // a thread's tile is kB sites wide and BY high
-constexpr unsigned long long kWaitNs = 2000000000ull;  // limit of a barrier wait
 constexpr int kBatch = kClusterBatch;
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) {
@@ -105,6 +104,14 @@ __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
   return t;
+}
+// Whether a wait since t0 is over: its limit has passed, which is reported, or another one's has (the
+// results are lost then, and the kernel ends without further waiting).
+__device__ __forceinline__ bool expired(unsigned long long t0, unsigned long long limit_ns, unsigned int *flags) {
+  if (*static_cast<volatile unsigned int *>(flags) & kFlagTimeout) return true;
+  if (global_ns() - t0 <= limit_ns) return false;
+  atomicOr(flags, kFlagTimeout);
+  return true;
 }
 __device__ __forceinline__ void mbar_arrive(unsigned bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
@@ -221,10 +228,7 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
     if (mbar_try(bar, parity)) return;
     const unsigned long long t0 = global_ns();
     for (unsigned it = 0; !mbar_try(bar, parity); ++it)
-      if ((it & 255u) == 255u && global_ns() - t0 > kWaitNs) {
-        atomicOr(a.flags, kFlagTimeout);
-        break;
-      }
+      if ((it & 255u) == 255u && expired(t0, a.wait_ns, a.flags)) break;
   };
   auto arrive_ends = [&]() {
     if (CS > 1) cluster_arrive();

@@ -133,10 +133,7 @@ __global__ void __launch_bounds__(WIDE ? 384 : kCxNarrow, 1) cluster_cplx_kernel
     } else if (!mbar_try(bar, phase)) {
       const unsigned long long t0 = global_ns();
       for (unsigned it = 0; !mbar_try(bar, phase); ++it)
-        if ((it & 255u) == 255u && global_ns() - t0 > kWaitNs) {
-          atomicOr(a.flags, kFlagTimeout);
-          break;
-        }
+        if ((it & 255u) == 255u && expired(t0, a.wait_ns, a.flags)) break;
     }
     phase ^= 1u;
   };

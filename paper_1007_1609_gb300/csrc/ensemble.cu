@@ -706,6 +706,7 @@ cudaError_t enqueue_iteration(cbdg_ensemble *e, double T, int M, double mix, dou
     c.dout = a.dout + o;
     c.nout = a.nout + o;
     c.flags = a.flags;
+    c.wait_ns = kWaitNs;
     c.mu = e->mu;
     c.coupling = e->U;
     c.hop = m.hop;

@@ -169,6 +169,7 @@ struct ClusterArgs {
   double *mu_ee;           // [ncols][M] or null
   double2 *mu_eh;          // [ncols][M][mom_stride] or null
   unsigned int *flags;
+  unsigned long long wait_ns;  // limit of a barrier wait
   double mu, coupling, hop, tol;  // hop: t of every bond; coupling: for dout
   int Lx, Ly, px, py, ncols, M, steps, mom_stride;
   int cluster, rows;       // CTAs per cluster, tile rows per CTA
@@ -193,6 +194,7 @@ struct AdjointClusterArgs {
   float4 *ck;              // [CTAs][M - 1][8][threads] the vectors j_0 .. j_{M-2} of a column
   float2 *acc;             // [CTAs][64][threads] gradient sums, zero before the first launch
   unsigned int *flags;
+  unsigned long long wait_ns;
   double mu, hop, scale;
   int stride, part;
   int Lx, Ly, px, py, ncols, M;
@@ -224,6 +226,7 @@ struct CplxClusterArgs {
   double *acc_n, *a_re;
   double2 *acc, *a_e, *a_h;
   unsigned int *flags;
+  unsigned long long wait_ns;
   double mu, tol;
   int mode, n_t, n_dirs;
   int Lx, Ly, px, py, ncols, M;

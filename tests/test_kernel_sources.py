@@ -17,3 +17,19 @@ def test_aligned_cluster_barriers_follow_a_warp_barrier(path):
     text = re.sub(r"//[^\n]*", "", open(path).read())
     for m in re.finditer(r'asm volatile\(\s*"barrier\.cluster\.[a-z.]*\.aligned', text):
         assert text[:m.start()].rstrip().endswith("__syncwarp();"), text[m.start():m.end()]
+
+
+def test_waits_of_the_on_chip_kernels_take_the_callers_limit():
+    """CBDG_OPT_WAIT_LIMIT_MS reaches every wait of the on-chip recursions: no
+    limit of their own, and every launch of a lattice passes the option on."""
+    for name in ("cluster.cuh", "cluster_cplx.cuh", "adjoint_cluster.cuh"):
+        text = open(os.path.join(CSRC, name)).read()
+        assert "kWaitNs" not in text, name
+        waits = re.findall(r"for \(unsigned it = 0; !mbar_try\(.*?;", text, re.S)
+        assert waits
+        assert text.count("expired(t0, a.wait_ns, a.flags)") == len(waits), name
+    api = open(os.path.join(CSRC, "api.cu")).read()
+    structs = re.findall(r"\b(ClusterArgs|CplxClusterArgs|AdjointClusterArgs) c\{\};", api)
+    assert len(structs) >= 4
+    # the general lattice's launches share one place that fills the rest of the arguments
+    assert api.count("c.wait_ns = static_cast<unsigned long long>(L->wait_ms) * 1000000ull;") == len(set(structs)) == 3
