@@ -2049,7 +2049,7 @@ cbdg_status cbdg_green_function(cbdg_lattice *L, const int32_t *sites, int32_t n
   CK(cudaMemcpyAsync(dE, he.data(), e_bytes, cudaMemcpyHostToDevice, L->stream));
   CK(launch_green_weights(n_E, M, kernel, lambda, dE, L->scal.as<double>(), W, L->stream));
   L->launches += 1;
-  // on the tensor cores, where the digit planes (half a gigabyte at most) fit the device
+  // on the tensor cores, where the digit planes fit the device (green_mma.cu says how large they get)
   const long long rows = static_cast<long long>(n_sites) * n_targets;
   bool digits = green_mma_wanted(rows, M, n_E);
   if (digits) {

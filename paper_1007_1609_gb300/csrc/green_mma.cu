@@ -2,7 +2,8 @@
 // (complex, FP64 in and out), on the tensor cores.
 //
 // FP64 units give two multiply-adds a clock and SM, the tensor cores a thousand.
-// Each operand row is scaled by a power of two and written as a 64-bit fixed-point number,
+// (Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 95 (2012): a matrix product as products of
+// exact slices.)  Each operand row is scaled by a power of two and written as a 64-bit fixed-point number,
 // eight signed base-256 digits (-128 .. 128) of bf16: x = 2^k sum_i d_i 2^(-7-8i).
 // Digits multiply exactly, a K-block of 128 terms adds them exactly in FP32 (of the
 // digit pairs (i, j) with the same i + j = d at most 8: 8 * 128 * 2^14 = 2^24), and
@@ -278,7 +279,10 @@ __global__ void __launch_bounds__(256, 1) digits_contract_kernel(int rows, int n
     }
 }
 
-constexpr size_t kPlaneBudget = size_t{256} << 20;  // bytes of the planes of the moments, and of the weights, at a time
+// Bytes of the planes of the moments, and of the weights, at a time: half a gigabyte together, but never
+// fewer than one tile of 64 rows each (smaller pieces would leave a CTA's tile empty and form the digits of
+// the moments again for each of them), so more above M = 131,072, up to 2 GB each at M = 2^20.
+constexpr size_t kPlaneBudget = size_t{256} << 20;
 
 struct Chunks {
   int kp, rows, energies;  // terms (padded), rows and energies at a time
