@@ -39,8 +39,8 @@ L, M, SEED = 128, 1024, 1001
 # per vector element and step: the stencil's 6 FMAs and half of a site's 6 product FMAs (FMA = 2 flops)
 FP64_FLOPS_PER_ELEMENT_STEP = 18.0
 FP32_FLOPS_PER_ELEMENT_STEP = 18.0
-# An FP32 adjoint advances an element twice (forward, reversed) at 12 flops, adds the source at 2 and
-# the gradient sums at 10.
+# An FP32 adjoint advances an element twice (forward and reverse recursion) at 12 flops and forms the
+# gradient sums at 12.
 ADJOINT_FLOPS_PER_ELEMENT_STEP = 36.0
 L2_FLUSH_BYTES = 256 << 20
 
@@ -611,8 +611,8 @@ def leg_adjoint(cbdg, wl, stream, hbm, fp32_peak=None):
             flops = ADJOINT_FLOPS_PER_ELEMENT_STEP * 2 * pg.N * pg.N * pg.M
             out["fp32_roofline"] = on_chip_roofline(
                 flops, dt * 1e3, fp32_peak,
-                "whole backward call: forward and reversed recursion, reverse recursion and gradient sums in the "
-                "registers of thread-block clusters")
+                "whole backward call: forward recursion, reverse recursion and gradient sums in the registers of "
+                "thread-block clusters, the forward vectors kept in HBM")
     return out
 
 
@@ -715,7 +715,7 @@ def leg_junction(cbdg, wl, torch, stream, hbm):
                                 "cluster_kernel (vectors in registers), one start site per layer")}
 
 
-def leg_green(cbdg, wl, torch, stream, fp64_peak=None):
+def leg_green(cbdg, wl, torch, stream):
     """Nonlocal Green's functions (gf1) around a vortex core of the 128x128
     d-wave lattice, M = 1024: 16 start sites (a 4x4 block at the core) x 256
     targets (a 16x16 block) x 512 energies in [-0.5a, 0.5a], device outputs.
@@ -854,7 +854,7 @@ def extra_legs(cbdg, wl, torch, stream, hbm, only=None, columns=4096, samples=25
         "adjoint": lambda: leg_adjoint(cbdg, wl, stream, hbm, fp32_peak=ap["fp32_fma"]["tflops"]),
         "currents": lambda: leg_currents(cbdg, wl, torch, stream, hbm),
         "junction": lambda: leg_junction(cbdg, wl, torch, stream, hbm),
-        "green": lambda: leg_green(cbdg, wl, torch, stream, fp64_peak=ap["fp64_fma"]["tflops"]),
+        "green": lambda: leg_green(cbdg, wl, torch, stream),
     }
     if only == "peaks":
         return {"peaks": ap}
