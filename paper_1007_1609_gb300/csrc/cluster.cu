@@ -37,13 +37,13 @@ int slots_of(const ClusterPlan &p) {
 // to 31 cycles (40 with tiles of 10, whose registers leave no room to reorder) for
 // each tile row of each of its warps, rounded up to its four schedulers, 500 for the latency of its barriers, edge
 // loads and sums, and 250 for every doubling of the cluster (all columns of 64 x 64, M = 512:
-// 4.54, 5.01 and 5.60 ms with tiles of 8 rows in clusters of 1, 2 and 4).  (The cycles were fitted
-// with plain sums; the compensated ones add about a tenth to every candidate and leave the order.)
-// High tiles exchange fewer edges per site and win where they fill the SM (4.54
-// against 4.66 ms with 4 rows there; 128 x 128, M = 512: 80.7 against 84.6 ms), tiles of 6
-// and 10 hold more sites per SM (96 x 96: 22.0 ms with 6 in one CTA against 31.8
-// and 34.9 with 4 and 8; 500 x 320 fits on chip only with 10), low ones leave more
-// warps to a lattice that leaves SMs idle (33 x 21, two iterations: 0.83 against 0.95 ms).
+// 4.37, 4.83 and 5.43 ms with tiles of 8 rows in clusters of 1, 2 and 4).  (The cycles were fitted
+// with plain sums; the compensated ones add up to a tenth to every candidate and leave the order.)
+// High tiles exchange fewer edges per site and win where they fill the SM (4.37
+// against 4.65 ms with 4 rows there; 128 x 128, M = 512: 76.1 against 82.5 ms), tiles of 6
+// and 10 hold more sites per SM (96 x 96: 21.1 ms with 6 in one CTA against 31.9
+// and 33.1 with 4 and 8; 500 x 320 fits on chip only with 10), low ones leave more
+// warps to a lattice that leaves SMs idle (33 x 21, two iterations: 0.82 against 0.93 ms).
 bool plan_cluster(int Lx, int Ly, int px, int py, int ncols, ClusterPlan *p) {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);

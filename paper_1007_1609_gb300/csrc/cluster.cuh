@@ -16,21 +16,21 @@
 // another tile, are computed in between.
 //
 // The three column sums of the doubling identities are formed per thread in
-// FP32 with compensation: the products of two rows of the tile, eight in each
-// half of the pair, in a chain of multiply-adds, the chains by compensated
-// addition (8 * 2^-24 of the sum of magnitudes in all).  The lanes of a warp are added in
+// FP32 with compensation: the products of four rows of the tile (two where it has
+// four), sixteen in each half of the pair, in a chain of multiply-adds, the chains by compensated
+// addition (16 * 2^-24 of the sum of magnitudes in all).  The lanes of a warp are added in
 // fixed point without rounding, kept per warp and step, and every 16 steps added
 // over the warps and CTAs (in FP64) and folded by one thread per step.  Root mean square
 // distance of the moments from FP64, over 33 x 21 .. 500 x 320 sites and M = 116 .. 2048: 0.69 (mu_ee)
 // and 0.80 (mu_eh) of the streamed kernels' (FP64 sums of the same vectors: 0.69 and 0.79; plain FP32
-// sums over tile and lanes: 0.71 and 0.82, and of the LDOS at a few sites 1.02, now 0.89).  The
-// compensated sums take a tenth of the time: 146 -> 160 ms for 128 x 128, M = 1024.
+// sums over tile and lanes: 0.71 and 0.82, and of the LDOS at a few sites 1.02, now 0.90).  Time of
+// 128 x 128, M = 1024: 146 ms with plain sums, 151 ms, 159 ms with chains of eight in all tiles.
 //
 // Bound: instruction issue and the FP32 pipe (fused multiply-adds with
 // three register operands run at two thirds of the pipe's rate).  Measured, one
-// map over all sites: 128 x 128, M = 1024: 160 ms (288 ms with three steps per
-// pass over HBM); 64 x 64, M = 512: 4.5 ms (14.6); 96 x 96: 22.0 ms (55.5); the
-// 75 x 90 torus: 18.8 ms (55.8, one step per pass); 11 start sites of a 100 x
+// map over all sites: 128 x 128, M = 1024: 151 ms (288 ms with three steps per
+// pass over HBM); 64 x 64, M = 512: 4.4 ms (14.6); 96 x 96: 21.1 ms (55.5); the
+// 75 x 90 torus: 17.6 ms (55.8, one step per pass); 11 start sites of a 100 x
 // 150 lattice, M = 2048: 1.3 ms (88 ms, one launch per step).
 #pragma once
 
@@ -127,30 +127,29 @@ __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
-// A thread's column sum v + e, |e| within the rounding of v (a sum of at most 1: |v| < 4).
-struct Sum {
-  float v = 0.f, e = 0.f;
-  __device__ __forceinline__ bool fits() const { return fabsf(v) < 4.f; }
+// A column sum (s and what its additions lost, r; both halves) in fixed point, in the mantissas of 12 + s,
+// units of 2^-20, and of 1.5 * 2^-19 + rest, units of 2^-42: without rounding down to the last of them while
+// |s| < 4 (a sum of at most 1).  head and tail add as integers.
+struct Fixed {
+  unsigned head0, head1, tail0, tail1;
+  __device__ __forceinline__ Fixed(F2 s, F2 r) {
+    const F2 t = f2add(s, f2bcast(12.f));
+    const F2 u = f2add(f2add(f2sub(s, f2sub(t, f2bcast(12.f))), r), f2bcast(0x1.8p-19f));
+    head0 = __float_as_uint(f2get(t, 0));
+    head1 = __float_as_uint(f2get(t, 1));
+    tail0 = __float_as_uint(f2get(u, 0));
+    tail1 = __float_as_uint(f2get(u, 1));
+  }
+  __device__ __forceinline__ bool fits() const {  // both heads in [8, 16)
+    return ((head0 ^ 0x41000000u) | (head1 ^ 0x41000000u)) < 0x00800000u;
+  }
+  __device__ __forceinline__ uint2 warp_sum() const {  // over the lanes of the warp
+    return make_uint2(__reduce_add_sync(0xffffffffu, head0 + head1), __reduce_add_sync(0xffffffffu, tail0 + tail1));
+  }
 };
-// The halves of s + r as one sum, exactly but for the rounding of e.
-__device__ __forceinline__ Sum halves(F2 s, F2 r) {
-  const float x = f2get(s, 0), y = f2get(s, 1);
-  Sum o;
-  o.v = __fadd_rn(x, y);
-  const float b = __fsub_rn(o.v, x);
-  o.e = __fadd_rn(__fadd_rn(__fsub_rn(x, __fsub_rn(o.v, b)), __fsub_rn(y, b)), __fadd_rn(f2get(r, 0), f2get(r, 1)));
-  return o;
-}
-// The sum of a warp's lanes in fixed point: each lane's value to units of 2^-20, then what is left of it
-// to units of 2^-42, which the mantissas of 12 + v and of 1.5 * 2^-19 + rest hold, added as integers.
-__device__ __forceinline__ uint2 warp_sum(const Sum &s) {
-  const float t = __fadd_rn(s.v, 12.f);
-  const float u = __fadd_rn(__fadd_rn(__fsub_rn(s.v, __fsub_rn(t, 12.f)), s.e), 0x1.8p-19f);
-  return make_uint2(__reduce_add_sync(0xffffffffu, __float_as_uint(t)), __reduce_add_sync(0xffffffffu, __float_as_uint(u)));
-}
 __device__ __forceinline__ long long warp_value(uint2 w) {  // in units of 2^-42
-  return static_cast<long long>(static_cast<int>(w.x - 32u * 0x41400000u)) * (1 << 22) +
-         static_cast<int>(w.y - 32u * 0x36400000u);
+  return static_cast<long long>(static_cast<int>(w.x - 64u * 0x41400000u)) * (1 << 22) +
+         static_cast<int>(w.y - 64u * 0x36400000u);
 }
 
 __device__ __forceinline__ float el(const Quad &v, int k) { return f2get(k < 2 ? v.lo : v.hi, k & 1); }
@@ -482,7 +481,7 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
           row(r, 1, er, el(hl, i + 2), el(hr, i + 2), 0, 0, 0, 0);
         }
       }
-      add_rows(k == 0);
+      if (BY == 4 || (k & 1)) add_rows(k < 2);  // the first chain is the sum
       publish_sides(ou, ov, 2 * k + 1, 2 * k + 2, k, wr);
     }
     arrive(bar_a);
@@ -517,10 +516,10 @@ __global__ void __launch_bounds__(Record<BY>::kThreads, 1) cluster_kernel(Cluste
     publish_ends(ou, 0, wr);
     publish_ends(ov, 1, wr);
     arrive_ends();
-    const Sum ta = halves(sa, ra), tb = halves(sb, rb), tc = halves(sc, rc);
-    A = warp_sum(ta);
-    B = warp_sum(tb);
-    C = warp_sum(tc);
+    const Fixed ta(sa, ra), tb(sb, rb), tc(sc, rc);
+    A = ta.warp_sum();
+    B = tb.warp_sum();
+    C = tc.warp_sum();
     // (|j_n| <= 1, unless the spectrum leaves [-1, 1])
     if (!ta.fits() || (2 * n + 1 < a.M && !(tb.fits() && tc.fits()))) atomicOr(a.flags, kFlagSpectrum);
   };

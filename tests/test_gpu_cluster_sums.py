@@ -3,9 +3,9 @@ of its vectors: on a torus without disorder the FP32 vectors of all start sites
 are translations of one another bit for bit, so the moments of different
 start sites differ by the rounding of the sums alone.
 
-Expected of sums with compensation: chains of at most eight products round
-with 0.7 * 2^-24 of the chain each (root mean square), independently, and
-nothing else rounds.  From the 32nd step on (moment 64) the weight lies on the whole lattice, 500 sites
+Expected of sums with compensation: chains of eight products (on these lattices,
+whose tiles have four or six rows, sixteen in some) round with 0.7 (0.9) * 2^-24 of
+the chain each (root mean square), independently, and nothing else rounds.  From the 32nd step on (moment 64) the weight lies on the whole lattice, 500 sites
 and more, in 63 chains at least: with amplitudes that vary by a factor of a few,
 2 * 0.7 * 2^-24 * 0.25 = 2.1e-8 at most for a moment.  Sums that round once or more at their own
 size (over the lanes of a warp, say) give 2 * 0.4 * 2^-24 * sqrt(2) = 6.7e-8 for the two
