@@ -21,8 +21,8 @@
 // M = 77 .. 512, in eps, t and Delta, and the time of 64 x 64, M = 512:
 //   reversed between pairs every 8 steps, products added one by one:  0.97 1.05 0.93   35.2 ms
 //   the same, every sum in FP64:                                      0.92 0.96 0.89
-//   stored vectors, products of a step first (this):                  0.91 0.93 0.84   37.2 ms
-//   with kFlush 32 or 16 in place of 64:                              0.92 0.94 0.84   40.2, 45.6 ms
+//   stored vectors, products of a step first (this):                  0.91 0.93 0.84   36.0 ms
+//   with kFlush 32 or 16 in place of 64:                              0.92 0.94 0.84   3 and 8 ms more
 //   stored vectors, every sum in FP64:                                0.86 0.86 0.79
 //
 // Bound: the FP32 pipe and instruction issue, 24 multiply-adds per site and step
@@ -36,6 +36,7 @@
 namespace cbdg {
 namespace {
 
+constexpr int kAhead = 4;    // steps that a vector is asked for ahead of its loads
 constexpr int kFlush = 64;   // steps between two moves of the sums to the scratch
 // A thread's record in shared memory, in quads: twice (double buffer) the edges
 // of j and of lam (Record<4>'s eight quads each), then its rows of 2 (eps - mu) / a
@@ -256,15 +257,20 @@ __global__ void __launch_bounds__(256, 1) adjoint_cluster_kernel(AdjointClusterA
       __stcs(ck + (static_cast<size_t>(n) * 8 + 4 + r) * blockDim.x, make_float4(at(v, r, 0), at(v, r, 1), at(v, r, 2), at(v, r, 3)));
     }
   };
+  // (volatile: at the head of the step among its reads of shared memory, not where the result is used: 37.2 ->
+  // 36.4 ms)
+  auto load_row = [](const float4 *p, F2 (&z)[2]) {
+    asm volatile("ld.global.cs.v2.b64 {%0, %1}, [%2];\n" : "=l"(z[0]), "=l"(z[1]) : "l"(p) : "memory");
+  };
+  // j_n of a warp, 32 lines, into L2: a line a lane (64 x 64, M = 512: 36.4 -> 36.0 ms)
+  auto prefetch = [&](int n) {
+    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(ck + (static_cast<size_t>(n) * 8 + (lane >> 2)) * blockDim.x - lane + (lane & 3) * 8));
+  };
   auto fetch = [&](int n, Tile4 &u, Tile4 &v) {
 #pragma unroll
     for (int r : {1, 2, 0, 3}) {
-      const float4 p = __ldcs(ck + (static_cast<size_t>(n) * 8 + r) * blockDim.x);
-      const float4 q = __ldcs(ck + (static_cast<size_t>(n) * 8 + 4 + r) * blockDim.x);
-      u[r][0] = f2pack(p.x, p.y);
-      u[r][1] = f2pack(p.z, p.w);
-      v[r][0] = f2pack(q.x, q.y);
-      v[r][1] = f2pack(q.z, q.w);
+      load_row(ck + (static_cast<size_t>(n) * 8 + r) * blockDim.x, u[r]);
+      load_row(ck + (static_cast<size_t>(n) * 8 + 4 + r) * blockDim.x, v[r]);
     }
   };
 
@@ -371,6 +377,7 @@ __global__ void __launch_bounds__(256, 1) adjoint_cluster_kernel(AdjointClusterA
       const Quad none{0, 0};
       F2 er[2], dr[2];
       if (m >= 2) fetch(m - 2, ou, ov);  // on its way during the step
+      if (m >= 2 + kAhead) prefetch(m - 2 - kAhead);
       wait(bar_a, phase);
       {
         const Quad hr = lds4(rt + rd), ll = lds4(lf + rd + fl), lr = lds4(rt + rd + fl);
