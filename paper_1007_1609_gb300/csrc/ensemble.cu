@@ -6,10 +6,10 @@
 // thread-block clusters (cluster.cuh): one launch per member, spread over eight
 // branches of the captured iteration so that one member's last columns and the
 // next one's first share the device.  256 members of sides 32 .. 96 (M = 512):
-// 1.81 s per iteration, against 5.3 s for the streaming kernel below, which is
+// 1.93 s per iteration, against 5.3 s for the streaming kernel below, which is
 // bound by the latency of its short rows at 55% of the copy bandwidth.  (One
 // launch over all members, the lattice changing inside the column loop, took
-// 2.10 s: the compiler then spends a quarter more instructions on a step.)
+// 1.16 times as long: the compiler then spends a quarter more instructions on a step.)
 //
 // The remaining members go to the streaming kernel, one persistent launch per
 // iteration.  Its work items are (sample, column slab of W start vectors), ordered largest

@@ -253,8 +253,9 @@ int best_threads(int XY, int M, int ncols) {
 
 // Always faster than the streamed kernels, which take 15 us a step at least and 20.7 operations a
 // site (61 x 45, M = 256: one column 4.2 -> 2.1 ms, 300: 5.8 -> 4.1; all of 56 x 56: 48.6 -> 41.7;
-// 60 x 60: 56.6 -> 50.7).  Lattices of 64 x 64 and more stay streamed: callers and tests rely on
-// their pass having a tile to choose.  Against the general kernel in shared memory (18 operations, no zeros beside the
+// 60 x 60: 56.6 -> 50.7).  Lattices of 64 x 64 and more stay with the streamed kernels, as the
+// header says of CBDG_OPT_RESIDENT, though those that fit would be faster here (64 x 64, M = 256: 77.3 -> 61.2
+// ms): their pass has a tile to choose.  Against the general kernel in shared memory (18 operations, no zeros beside the
 // lattice; W_general its slab width) by the operations of an SM: 16 x 16 stays there (0.54 ms, 0.62
 // here), 32 x 32 periodic does not (4.94 -> 4.16), nor 40 x 40 (12.2 -> 11.6).
 bool plan_resident_uniform(int Lx, int Ly, int px, int py, int ncols, int M, int W_general) {
