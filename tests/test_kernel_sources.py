@@ -33,3 +33,13 @@ def test_waits_of_the_on_chip_kernels_take_the_callers_limit():
     assert len(structs) >= 4
     # the general lattice's launches share one place that fills the rest of the arguments
     assert api.count("c.wait_ns = static_cast<unsigned long long>(L->wait_ms) * 1000000ull;") == len(set(structs)) == 3
+
+
+def test_destroy_frees_every_buffer_of_a_lattice():
+    api = open(os.path.join(CSRC, "api.cu")).read()
+    struct = api[api.index("struct cbdg_lattice {"):]
+    struct = re.sub(r"//[^\n]*", "", struct[:struct.index("\n};")])
+    members = [m for line in re.findall(r"\bDBuf ([^;()]*);", struct) for m in re.findall(r"\w+", line)]
+    destroy = api[api.index("cbdg_status cbdg_destroy("):]
+    freed = re.findall(r"&L->(\w+)", destroy[:destroy.index("b->release()")])
+    assert len(members) > 40 and sorted(members) == sorted(freed)
