@@ -106,8 +106,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 // Whether a wait since t0 is over: its limit has passed, which is reported, or another one's has (the
-// results are lost then, and the kernel ends without further waiting).
-__device__ __forceinline__ bool expired(unsigned long long t0, unsigned long long limit_ns, unsigned int *flags) {
+// results are lost then, and the kernel ends without further waiting).  A call of its own: inlined at each
+// wait it changes the step's schedule (75 x 90 torus: 17.6 ms, 16.7 so).
+__device__ __noinline__ bool expired(unsigned long long t0, unsigned long long limit_ns, unsigned int *flags) {
   if (*static_cast<volatile unsigned int *>(flags) & kFlagTimeout) return true;
   if (global_ns() - t0 <= limit_ns) return false;
   atomicOr(flags, kFlagTimeout);
