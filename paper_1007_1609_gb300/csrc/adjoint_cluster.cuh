@@ -21,7 +21,7 @@
 // M = 77 .. 512, in eps, t and Delta, and the time of 64 x 64, M = 512:
 //   reversed between pairs every 8 steps, products added one by one:  0.97 1.05 0.93   35.2 ms
 //   the same, every sum in FP64:                                      0.92 0.96 0.89
-//   stored vectors, products of a step first (this):                  0.91 0.93 0.84   36.0 ms
+//   stored vectors, products of a step first (this):                  0.91 0.93 0.84   36.5 ms
 //   with kFlush 32 or 16 in place of 64:                              0.92 0.94 0.84   3 and 8 ms more
 //   stored vectors, every sum in FP64:                                0.86 0.86 0.79
 //

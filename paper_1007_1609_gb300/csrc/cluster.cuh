@@ -30,7 +30,7 @@
 // three register operands run at two thirds of the pipe's rate).  Measured, one
 // map over all sites: 128 x 128, M = 1024: 151 ms (288 ms with three steps per
 // pass over HBM); 64 x 64, M = 512: 4.4 ms (14.6); 96 x 96: 21.1 ms (55.5); the
-// 75 x 90 torus: 17.6 ms (55.8, one step per pass); 11 start sites of a 100 x
+// 75 x 90 torus: 16.8 ms (55.8, one step per pass); 11 start sites of a 100 x
 // 150 lattice, M = 2048: 1.3 ms (88 ms, one launch per step).
 #pragma once
 

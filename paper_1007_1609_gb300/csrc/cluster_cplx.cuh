@@ -26,7 +26,7 @@
 // Both start vectors in one thread read the coefficients once for two (50 quads a
 // vector) but leave one warp a scheduler: 75.3 ms for the currents.
 // Streamed kernel -> this one: d-wave vortex lattices, 96 x 96, 512 start sites,
-// M = 1024: 59.8 -> 32.4 ms; bond currents of 64 x 64, M = 512: 75.1 -> 54.0 ms;
+// M = 1024: 59.8 -> 32.4 ms; bond currents of 64 x 64, M = 512: 75.1 -> 52.5 ms;
 // Green's functions of 128 x 128, 16 x 256 sites, M = 1024: 17.0 -> 9.8 ms (3.4 of them the
 // contraction with the energies).  The sums are those of the streamed kernels in
 // their order: the same moments bit for bit.  (Starting from e u - u_old instead of
